@@ -178,9 +178,10 @@ struct Server {
     const int64_t blocks = std::min<int64_t>(152 * 4, (K + kBvpThreads - 1) / kBvpThreads);
     int64_t b = nf * nz * ny * pitch * 2 * ts;                          // grid
     b += nmax * (rec + 8 + 15 * 8) + 3 * nbins * 4;                      // records, bins, staging
-    b += blocks * kBvpThreads * nz * (3 * 16 + 3 * 8 + 2 * ts);          // solve workspace
+    // solve workspace (the tiled solve, which takes none, applies to every column up to one pass of blocks)
+    if (nz > 128 || blocks >= 152 * 3) b += blocks * kBvpThreads * nz * (3 * 16 + 3 * 8 + 2 * ts);
     b += 3 * nz * K * 2 * ts + 12 * K * 2 * ts;                          // kbuf, kaux
-    b += nkx * (ny / 2 + 1) * nz * 4 * 8;                                // factorisation table (FP64)
+    b += nkx * (ny / 2 + 1) * (nz * 48 + 14 * 8);                        // the solve's table
     // partial sums of the tile-gather interpolation (forces only, or equal supports with the
     // spectral curl): slots of the tiles a support can overlap x fields x particles
     const int64_t ifields = route == DPS_TORQUE_NONE ? 3

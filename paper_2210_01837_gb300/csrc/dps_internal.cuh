@@ -117,7 +117,8 @@ struct KTabs {
   void* cmat;      // [N][N]     forward DCT-I C[n][j] (correction coefficients in the tiled backward)
   void* kbuf;      // [3][N][K]  Chebyshev coefficients per wavenumber (forces, then DP velocity)
   void* kaux;      // [12][K]    wall-correction amplitudes per wavenumber
-  double* fac;     // [N][4][KP] factorisation of the banded systems per (kx, |ky|) (FP64), or null
+  double* fac;     // factorisation of the banded systems per (kx, |ky|): the tiled solve's table (solve.cu), or
+                   // [N][4][KP] for the thread-per-wavenumber solve (bvp.cu); null without one
   int64_t KP;      // nkx (ny/2 + 1)
   unsigned char* bimg_f;  // tensor-core transforms: B operands of every K step (forward, backward)
   unsigned char* bimg_b;
@@ -155,7 +156,8 @@ struct Plan {
   alignas(64) unsigned char interp_tmap[128];  // CUtensorMap of the grid for the staged interpolation
   int interp_tma;       // interp_tmap holds a valid map
   int col_tma_rows;     // rows per TMA box of that pass
-  int bvp_blocks_max;   // persistent solve blocks the workspace was allocated for
+  int bvp_blocks_max;   // most persistent solve blocks: what the GPU holds at once (and the workspace was allocated for)
+  int solve_tile;       // the tiled solve (solve.cu) runs: a factorisation table and nz <= 128
   int interp_tile;      // interpolation variant: 0 warp per particle, 1 tile gather, 2 staged grid (where they apply)
   int cheb_tc;          // forward Chebyshev transform on the tensor cores (tcgen05, mixed precision)
   int cheb_tc_bwd;      // backward Chebyshev transform on the tensor cores (spectral-curl torques)
@@ -287,6 +289,12 @@ template <typename T> int bvp_prepare(Plan& p);
 // the factorisation table of the FP64 solve (allocated and filled at plan creation); DPS_ERR_OOM
 // leaves the plan on the factorise-as-you-go solve
 dps_status bvp_factor_table(Plan& p);
+// the tiled solve (solve.cu): where it applies, its resident grid (0 on a CUDA error), its table (allocated
+// and filled; as bvp_factor_table), and its launcher
+bool solve_tile_applies(const Geometry& g, int precision);
+template <typename T> int solve_tile_prepare(const Plan& p);
+dps_status solve_tile_table(Plan& p);
+template <typename T> void launch_solve_tile(const Plan& p, int kx0, int w, cudaStream_t s);
 // the tensor-core forward Chebyshev transform: readiness (sets cheb_tc where it applies; 0 on a CUDA
 // error), its launcher, and its accumulator width (nz rounded up to 16)
 int cheb_tc_prepare(Plan& p);

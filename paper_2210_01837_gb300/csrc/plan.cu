@@ -316,13 +316,7 @@ dps_status allocate(Plan* p) {
   if (!alloc((void**)&p->zrange, 2 * sizeof(int))) return DPS_ERR_OOM;
   if (!alloc((void**)&p->status, sizeof(int))) return DPS_ERR_OOM;
   if (cudaMemset(p->status, 0, sizeof(int)) != cudaSuccess) return DPS_ERR_CUDA;
-  p->bvp_blocks = bvp_occupancy_blocks<T>(*p);
   const int64_t K = (int64_t)g.nkx * g.ny;
-  const int64_t need_blocks = (K + kBvpThreads - 1) / kBvpThreads;
-  if (p->bvp_blocks > need_blocks) p->bvp_blocks = (int)std::max<int64_t>(1, need_blocks);
-  p->bvp_blocks_max = p->bvp_blocks;
-  p->ws_bytes = (int64_t)p->bvp_blocks * kBvpThreads * (int64_t)bvp_slot_bytes<T>(*p);
-  if (!alloc(&p->ws, (size_t)p->ws_bytes)) return DPS_ERR_OOM;
   if (!alloc(&p->kt.kbuf, 3 * (size_t)g.nz * (size_t)K * sizeof(cplx<T>))) return DPS_ERR_OOM;
   if (!alloc(&p->kt.kaux, 12 * (size_t)K * sizeof(cplx<T>))) return DPS_ERR_OOM;
   if (!bvp_prepare<T>(*p)) return DPS_ERR_INVALID_ARG;
@@ -343,6 +337,19 @@ dps_status allocate(Plan* p) {
       if (ft == DPS_ERR_CUDA) return ft;
     }
   }
+  // the tiled solve keeps its sweeps in shared memory; the thread-per-wavenumber solves need a workspace
+  p->solve_tile = p->kt.fac && solve_tile_applies(g, p->precision) ? 1 : 0;
+  if (p->solve_tile) {
+    p->bvp_blocks = solve_tile_prepare<T>(*p);
+    if (p->bvp_blocks < 1) return DPS_ERR_CUDA;
+  } else {
+    p->bvp_blocks = bvp_occupancy_blocks<T>(*p);
+    const int64_t need_blocks = (K + kBvpThreads - 1) / kBvpThreads;
+    if (p->bvp_blocks > need_blocks) p->bvp_blocks = (int)std::max<int64_t>(1, need_blocks);
+    p->ws_bytes = (int64_t)p->bvp_blocks * kBvpThreads * (int64_t)bvp_slot_bytes<T>(*p);
+    if (!alloc(&p->ws, (size_t)p->ws_bytes)) return DPS_ERR_OOM;
+  }
+  p->bvp_blocks_max = p->bvp_blocks;
   // the tile-gather interpolation's partial sums (where it applies; a variant the autotuner tries)
   if (const size_t iv = interp_tile_values(g, p->max_n)) {
     if (!alloc(&p->ipart, iv * sizeof(T))) return DPS_ERR_OOM;
