@@ -182,6 +182,7 @@ struct Server {
     if (nz > 128 || blocks >= 152 * 3) b += blocks * kBvpThreads * nz * (3 * 16 + 3 * 8 + 2 * ts);
     b += 3 * nz * K * 2 * ts + 12 * K * 2 * ts;                          // kbuf, kaux
     b += nkx * (ny / 2 + 1) * (nz * 48 + 14 * 8);                        // the solve's table
+    if (ts == 8) b += nkx * (ny / 2 + 1) * nz * 16 + 256 * nz * nz;      // the folded transforms' tables
     // partial sums of the tile-gather interpolation (forces only, or equal supports with the
     // spectral curl): slots of the tiles a support can overlap x fields x particles
     const int64_t ifields = route == DPS_TORQUE_NONE ? 3

@@ -40,13 +40,6 @@ namespace dps {
 
 namespace {
 
-// thread i of a chunk (columns [kx0, kx0 + w), every ky) -> wavenumber column; kidx = kyi*nkx + kxi
-__device__ __forceinline__ int64_t chunk_kidx(const Geometry& g, int64_t i, int kx0, int w) {
-  const unsigned ii = (unsigned)i;  // total wavenumbers < 2^31
-  const int kyi = (int)(ii / (unsigned)w);
-  return (int64_t)kyi * g.nkx + kx0 + (int)(ii - (unsigned)kyi * (unsigned)w);
-}
-
 // per-block wavenumber table of the tiled kernels: grid column offset, kbuf index, k/2 components
 struct KTile {
   int col[64];
@@ -1565,7 +1558,9 @@ void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s) {
   cplx<T>* kbuf = reinterpret_cast<cplx<T>*>(p.kt.kbuf);
   cplx<T>* kaux = reinterpret_cast<cplx<T>*>(p.kt.kaux);
   const LaneCfg fc = fwd_lane_cfg<T>(g);
-  if (part == 0 && sizeof(T) == 4 && p.cheb_tc) {
+  if (part != 1 && p.cheb_fold) {
+    launch_cheb_fold(p, part == 2, kx0, w, s);
+  } else if (part == 0 && sizeof(T) == 4 && p.cheb_tc) {
     launch_cheb_fwd_tc(p, kx0, w, s);
   } else if (part == 0 && fc.threads > 0) {
     const unsigned lb = (unsigned)((total + kLaneK - 1) / kLaneK);

@@ -65,6 +65,13 @@ __device__ __forceinline__ cplx<double> cdiv(cplx<double> a, cplx<double> b) {
   return mk<double>((a.x * b.x + a.y * b.y) / den, (a.y * b.x - a.x * b.y) / den);
 }
 
+// thread i of a chunk (columns [kx0, kx0 + w), every ky) -> wavenumber column; kidx = kyi*nkx + kxi
+__device__ __forceinline__ int64_t chunk_kidx(const Geometry& g, int64_t i, int kx0, int w) {
+  const unsigned ii = (unsigned)i;  // total wavenumbers < 2^31
+  const int kyi = (int)(ii / (unsigned)w);
+  return (int64_t)kyi * g.nkx + kx0 + (int)(ii - (unsigned)kyi * (unsigned)w);
+}
+
 struct KInfo {
   int kxi, kyi;
   bool nyq, zero;

@@ -120,6 +120,8 @@ struct KTabs {
   double* fac;     // factorisation of the banded systems per (kx, |ky|): the tiled solve's table (solve.cu), or
                    // [N][4][KP] for the thread-per-wavenumber solve (bvp.cu); null without one
   int64_t KP;      // nkx (ny/2 + 1)
+  double* fold;    // folded transforms (cheb_fold.cu): forward and backward part matrices, then the coefficients of
+                   // e^{-k zeta} and zeta e^{-k zeta} [N][KP]; null where they do not apply
   unsigned char* bimg_f;  // tensor-core transforms: B operands of every K step (forward, backward)
   unsigned char* bimg_b;
   int npad, cpad;
@@ -161,6 +163,7 @@ struct Plan {
   int interp_tile;      // interpolation variant: 0 warp per particle, 1 tile gather, 2 staged grid (where they apply)
   int cheb_tc;          // forward Chebyshev transform on the tensor cores (tcgen05, mixed precision)
   int cheb_tc_bwd;      // backward Chebyshev transform on the tensor cores (spectral-curl torques)
+  int cheb_fold;        // Chebyshev transforms by folding (double precision, nz - 1 a multiple of 8)
   int cheb_tc_bwd_parts;  // launches of the backward transform (output planes split beyond 96 nodes)
   int cheb_tc_grid;     // persistent blocks of that kernel
   int inject;           // failure injection of the next apply (dpstokes_debug_inject)
@@ -301,6 +304,12 @@ int cheb_tc_prepare(Plan& p);
 void launch_cheb_fwd_tc(const Plan& p, int kx0, int w, cudaStream_t s);
 void launch_cheb_bwd_tc(const Plan& p, int kx0, int w, cudaStream_t s);
 int cheb_tc_np(const Geometry& g);
+// the folded transforms (cheb_fold.cu): where they apply, the bytes of their tables, their preparation (DPS_ERR_OOM
+// leaves the plan on the lane kernels) and launcher
+bool cheb_fold_applies(const Plan& p);
+size_t cheb_fold_bytes(const Geometry& g);
+dps_status cheb_fold_prepare(Plan& p);
+void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t s);
 size_t cheb_tc_image_bytes(const Geometry& g, bool backward);
 template <typename T> size_t bvp_slot_bytes(const Plan& p);
 template <typename T> int fft_smem_ok(Plan& p);

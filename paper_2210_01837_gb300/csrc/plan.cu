@@ -166,7 +166,7 @@ void free_plan(Plan* p) {
                   p->kt.ct, p->kt.dct,
                   p->kt.ict, p->kt.icdt, p->kt.sdt, p->kt.bandT, p->kt.cmat, p->kt.kbuf, p->kt.kaux, p->grid, p->records, p->bin_of, p->bin_count, p->bin_start,
                   p->bin_cursor, p->sorted, p->zrange, p->status, p->ws, p->stage_in, p->stage_out, p->ipart,
-                  p->kt.fac, p->kt.bimg_f, p->kt.bimg_b};
+                  p->kt.fac, p->kt.fold, p->kt.bimg_f, p->kt.bimg_b};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete p;
@@ -327,6 +327,11 @@ dps_status allocate(Plan* p) {
     const int v = atoi(e);
     p->cheb_tc = p->cheb_tc && (v & 1);
     p->cheb_tc_bwd = p->cheb_tc_bwd && (v & 2);
+  }
+  if (cheb_fold_applies(*p)) {
+    const dps_status fs = cheb_fold_prepare(*p);
+    if (fs == DPS_ERR_CUDA) return fs;
+    p->cheb_fold = fs == DPS_OK ? 1 : 0;
   }
   // factorisation table of the FP64 solve (per (kx, |ky|), filled on the legacy stream): without
   // the memory for it the solve factorises as it goes; DPS_SOLVE_TABLE=0 chooses that by hand
