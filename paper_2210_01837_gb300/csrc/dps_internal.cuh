@@ -284,7 +284,6 @@ bool encode_interp_tmap(Plan& p);
 size_t interp_tile_values(const Geometry& g, int64_t max_n);
 template <typename T> void launch_fft_rows(const Plan& p, int dir, cudaStream_t s);
 template <typename T> void launch_fft_cols(const Plan& p, int dir, int kxs, int kxe, cudaStream_t s);
-template <typename T> int fft_col_width(const Plan& p);
 // part 0 Chebyshev forward, 1 FP64 solve, 2 backward; columns [kx0, kx0 + w) of every ky
 template <typename T> void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s);
 template <typename T> int bvp_occupancy_blocks(const Plan& p);
@@ -312,7 +311,11 @@ dps_status cheb_fold_prepare(Plan& p);
 void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t s);
 size_t cheb_tc_image_bytes(const Geometry& g, bool backward);
 template <typename T> size_t bvp_slot_bytes(const Plan& p);
-template <typename T> int fft_smem_ok(Plan& p);
+// the passes' kernels' shared-memory limits and default variants
+template <typename T> bool fft_rows_allow();
+template <typename T> bool fft_cols_allow();
+template <typename T> bool fft_rows_default(Plan& p);
+template <typename T> bool fft_cols_default(Plan& p);
 // column block 2^lcw and variant of the y-FFT pass (reg: 0 shared-memory-staged, 1 register-staged,
 // 2 register-staged with cp.async prefetch, 3 register-staged with TMA prefetch); 0 if it does not fit
 template <typename T> int fft_set_col_width(Plan& p, int lcw, int reg);

@@ -17,14 +17,20 @@
 // buffer, the first stage reading HBM and the last writing it directly (described further below);
 // for the column pass also with a second buffer that receives the next unit, by cp.async or by
 // TMA box loads on an mbarrier.
-// The plan picks the variant per pass (default rule at fft_smem_ok, or autotuned / set by hand).
+// The plan picks the variant per pass (default rules at fft_rows_default and
+// fft_cols_default, or autotuned / set by hand).
 // Each 1D transform is a self-sorting (Stockham) mixed-radix FFT in shared memory written from the
 // textbook formulation: stage s with radix R and span Ns multiplies input j + r n/R by
 // W_{Ns R}^{(j mod Ns) r}, applies an R-point DFT, and stores to (j / Ns) Ns R + (j mod Ns) + r Ns.
-// Radices 16, 12 (as 4 x 4 and 4 x 3), 8, 4, 2 (hand-written butterflies) and 3, 5, 7 (direct DFT
-// with exact constants).  Twiddles W_n^t = exp(-2 pi i t/n) come from a table built in double
-// precision on the host; the register-staged column passes read per-stage rows W_{Ns R}^{k r}
-// instead (one contiguous row per butterfly).
+// Radices 16 (as 4 x 4), 9 (as 3 x 3), 8, 4, 2, the odd primes 3, 5, 7, and the coprime products 15, 14, 12, 10
+// and 6 (Good's mapping, no inner twiddles).  The products save stages, each a trip through shared memory
+// and a barrier: 630 = 10 9 7 instead of 7 5 3 3 2 (rows 561 -> 412, columns 728 -> 478 us at 65 nodes), 2700 =
+// 15 15 12 (columns 4.34 -> 2.33 ms at 19 nodes, 4 columns a block instead of 2), 384 x 384 x 97 in double
+// (384 = 16 12 2 by the cheaper radix 12) rows 2.87 -> 2.44 ms.  Twiddles W_n^t = exp(-2 pi i t/n) come from a
+// table built in double precision on the host; the register-staged column passes read per-stage rows
+// W_{Ns R}^{k r} instead (one contiguous row per butterfly).
+#pragma once
+
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -166,59 +172,108 @@ template <typename T, int DIR> struct Dft<T, 16, DIR> {
   }
 };
 
+// Odd prime R: X_k and X_{R-k} from the sums and differences of conjugate inputs,
+// X_k = v_0 + sum_j cos(2 pi j k / R) (v_j + v_{R-j}) +- i sum_j sin(2 pi j k / R) (v_j - v_{R-j}),
+// half the multiply-adds of the direct sums
 template <typename T, int R, int DIR>
-__device__ __forceinline__ void dft_direct(cplx<T>* v) {
-  cplx<T> out[R];
+__device__ __forceinline__ void dft_odd(cplx<T>* v) {
+  constexpr int h = R / 2;
+  cplx<T> s[h + 1], d[h + 1];
 #pragma unroll
-  for (int k = 0; k < R; ++k) {
-    cplx<T> acc = v[0];
-#pragma unroll
-    for (int r = 1; r < R; ++r) {
-      const int m = (r * k) % R;
-      const cplx<T> w = mk<T>(root_cos<T, R>(m), DIR > 0 ? root_sin<T, R>(m) : -root_sin<T, R>(m));
-      acc = acc + v[r] * w;
-    }
-    out[k] = acc;
+  for (int j = 1; j <= h; ++j) {
+    s[j] = v[j] + v[R - j];
+    d[j] = v[j] - v[R - j];
   }
+  const cplx<T> v0 = v[0];
 #pragma unroll
-  for (int k = 0; k < R; ++k) v[k] = out[k];
+  for (int j = 1; j <= h; ++j) v[0] = v[0] + s[j];
+#pragma unroll
+  for (int k = 1; k <= h; ++k) {
+    cplx<T> a = v0, b = mk<T>((T)0, (T)0);
+#pragma unroll
+    for (int j = 1; j <= h; ++j) {
+      const int m = (j * k) % R;
+      a = a + scl(s[j], root_cos<T, R>(m));
+      b = b + scl(d[j], (T)DIR * root_sin<T, R>(m));
+    }
+    b = mul_i(b);
+    v[k] = a + b;
+    v[R - k] = a - b;
+  }
 }
 
 template <typename T, int DIR> struct Dft<T, 3, DIR> {
-  static __device__ __forceinline__ void run(cplx<T>* v) { dft_direct<T, 3, DIR>(v); }
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_odd<T, 3, DIR>(v); }
 };
 template <typename T, int DIR> struct Dft<T, 5, DIR> {
-  static __device__ __forceinline__ void run(cplx<T>* v) { dft_direct<T, 5, DIR>(v); }
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_odd<T, 5, DIR>(v); }
 };
 template <typename T, int DIR> struct Dft<T, 7, DIR> {
-  static __device__ __forceinline__ void run(cplx<T>* v) { dft_direct<T, 7, DIR>(v); }
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_odd<T, 7, DIR>(v); }
 };
 
-// 12-point DFT as 4 x 3: x[3 a + b] -> X[c + 4 d]; inner DFT4 over a, twiddle W12^(b c), outer DFT3 over b
+// A B points, A and B coprime (Good's mapping: no twiddles): input (B a + A b) mod A B takes DFT_A over a,
+// then DFT_B over b; output k has k mod A = c, k mod B = d
+template <typename T, int A, int B, int DIR>
+__device__ __forceinline__ void dft_coprime(cplx<T>* v) {
+  constexpr int N = A * B;
+  cplx<T> y[B][A];
+#pragma unroll
+  for (int b = 0; b < B; ++b) {
+#pragma unroll
+    for (int a = 0; a < A; ++a) y[b][a] = v[(B * a + A * b) % N];
+    Dft<T, A, DIR>::run(y[b]);
+  }
+#pragma unroll
+  for (int c = 0; c < A; ++c) {
+    cplx<T> w[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) w[b] = y[b][c];
+    Dft<T, B, DIR>::run(w);
+#pragma unroll
+    for (int k = c; k < N; k += A) v[k] = w[k % B];
+  }
+}
+template <typename T, int DIR> struct Dft<T, 6, DIR> {
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_coprime<T, 2, 3, DIR>(v); }
+};
+template <typename T, int DIR> struct Dft<T, 10, DIR> {
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_coprime<T, 2, 5, DIR>(v); }
+};
 template <typename T, int DIR> struct Dft<T, 12, DIR> {
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_coprime<T, 4, 3, DIR>(v); }
+};
+template <typename T, int DIR> struct Dft<T, 14, DIR> {
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_coprime<T, 2, 7, DIR>(v); }
+};
+template <typename T, int DIR> struct Dft<T, 15, DIR> {
+  static __device__ __forceinline__ void run(cplx<T>* v) { dft_coprime<T, 3, 5, DIR>(v); }
+};
+
+// 9-point DFT as 3 x 3: x[3 a + b] -> X[c + 3 d]; inner DFT3 over a, twiddle W9^(b c), outer DFT3 over b
+template <typename T, int DIR> struct Dft<T, 9, DIR> {
   static __device__ __forceinline__ void run(cplx<T>* v) {
-    const T h = (T)0.5, s3 = (T)0.86602540378443865, sg = (T)DIR;  // cos/sin of 30 and 60 degrees
-    cplx<T> y[3][4];
+    const T sg = (T)DIR;
+    const T c1 = (T)0.76604444311897804, s1 = (T)0.64278760968653933;   // 40 degrees
+    const T c2 = (T)0.17364817766693035, s2 = (T)0.98480775301220806;   // 80 degrees
+    const T c4 = (T)-0.93969262078590838, s4 = (T)0.34202014332566873;  // 160 degrees
+    cplx<T> y[3][3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      cplx<T> w[4] = {v[b], v[3 + b], v[6 + b], v[9 + b]};
-      Dft<T, 4, DIR>::run(w);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) y[b][c] = w[c];
+      for (int a = 0; a < 3; ++a) y[b][a] = v[3 * a + b];
+      Dft<T, 3, DIR>::run(y[b]);
     }
-    // W12^m = (cos(2 pi m / 12), DIR sin(2 pi m / 12)) for m = b c
-    y[1][1] = y[1][1] * mk<T>(s3, sg * h);
-    y[1][2] = y[1][2] * mk<T>(h, sg * s3);
-    y[1][3] = rot_quarter<T, DIR>(y[1][3]);
-    y[2][1] = y[2][1] * mk<T>(h, sg * s3);
-    y[2][2] = y[2][2] * mk<T>(-h, sg * s3);
-    y[2][3] = mk<T>(-y[2][3].x, -y[2][3].y);
+    y[1][1] = y[1][1] * mk<T>(c1, sg * s1);
+    y[1][2] = y[1][2] * mk<T>(c2, sg * s2);
+    y[2][1] = y[2][1] * mk<T>(c2, sg * s2);
+    y[2][2] = y[2][2] * mk<T>(c4, sg * s4);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < 3; ++c) {
       cplx<T> w[3] = {y[0][c], y[1][c], y[2][c]};
       Dft<T, 3, DIR>::run(w);
 #pragma unroll
-      for (int d = 0; d < 3; ++d) v[c + 4 * d] = w[d];
+      for (int d = 0; d < 3; ++d) v[c + 3 * d] = w[d];
     }
   }
 };
@@ -283,6 +338,11 @@ template <typename T, int DIR, class In>
 __device__ __forceinline__ void fft_first(cplx<T>* buf, const FftPlan& fp, int lbatch, const In& in) {
   switch (fp.radix[0]) {
     case 16: stage_first<T, 16, DIR>(buf, fp.n, lbatch, in); break;
+    case 15: stage_first<T, 15, DIR>(buf, fp.n, lbatch, in); break;
+    case 14: stage_first<T, 14, DIR>(buf, fp.n, lbatch, in); break;
+    case 10: stage_first<T, 10, DIR>(buf, fp.n, lbatch, in); break;
+    case 9: stage_first<T, 9, DIR>(buf, fp.n, lbatch, in); break;
+    case 6: stage_first<T, 6, DIR>(buf, fp.n, lbatch, in); break;
     case 12: stage_first<T, 12, DIR>(buf, fp.n, lbatch, in); break;
     case 8: stage_first<T, 8, DIR>(buf, fp.n, lbatch, in); break;
     case 4: stage_first<T, 4, DIR>(buf, fp.n, lbatch, in); break;
@@ -305,6 +365,11 @@ __device__ cplx<T>* fft_rest(cplx<T>* b0, cplx<T>* b1, const FftPlan& fp, int lb
     const unsigned long long mg = fp.magic[s];
     switch (R) {
       case 16: stage<T, 16, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
+      case 15: stage<T, 15, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
+      case 14: stage<T, 14, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
+      case 10: stage<T, 10, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
+      case 9: stage<T, 9, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
+      case 6: stage<T, 6, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
       case 12: stage<T, 12, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
       case 8: stage<T, 8, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
       case 4: stage<T, 4, DIR>(in, out, fp.n, Ns, mg, lbatch, tw); break;
@@ -641,18 +706,32 @@ __device__ __forceinline__ void reg_stage(const FftPlan& fp, int s, int Ns, int 
   if (act) store_all<T, R>(v, dst, ob, Ns, b);
 }
 
-template <typename T, int DIR, bool ST, class Src, class Dst>
+// ODD: the factorisation may hold radices with a factor 5 or 7, or 9.  Without them the column kernels keep
+// to their 64 registers; with them they spill a few values at the widest radices, which costs 2^a 3^b
+// columns 5 to 9 % (768 rows: 541 -> 590 us).
+template <typename T, int DIR, bool ST, bool ODD, class Src, class Dst>
 __device__ __forceinline__ void reg_stage_any(const FftPlan& fp, int s, int Ns, int lb, const cplx<T>* tw,
                                               const Src& src, const Dst& dst, bool barrier) {
-  switch (fp.radix[s]) {
+  const int R = fp.radix[s];
+  if constexpr (ODD) {
+    switch (R) {
+      case 15: reg_stage<T, 15, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); return;
+      case 14: reg_stage<T, 14, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); return;
+      case 10: reg_stage<T, 10, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); return;
+      case 9: reg_stage<T, 9, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); return;
+      case 7: reg_stage<T, 7, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); return;
+      case 5: reg_stage<T, 5, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); return;
+      default: break;
+    }
+  }
+  switch (R) {
     case 16: reg_stage<T, 16, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
     case 12: reg_stage<T, 12, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
     case 8: reg_stage<T, 8, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
+    case 6: reg_stage<T, 6, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
     case 4: reg_stage<T, 4, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
     case 2: reg_stage<T, 2, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
-    case 3: reg_stage<T, 3, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
-    case 5: reg_stage<T, 5, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
-    default: reg_stage<T, 7, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
+    default: reg_stage<T, 3, DIR, ST>(fp, s, Ns, lb, tw, src, dst, barrier); break;
   }
 }
 
@@ -662,7 +741,7 @@ __device__ __forceinline__ void reg_stage_any(const FftPlan& fp, int s, int Ns, 
 // PW: pad elements per 16 in the shared buffer (1; 2 keeps float pairs 16-byte aligned for cp.async).
 // ST: tw is the stage-twiddle table (column passes) rather than the length-n table (row passes,
 // whose tighter register budget the row loads do not fit)
-template <typename T, int DIR, bool DST_SMEM, bool ST, int PW = 1, int SH = 4, class Src, class Dst>
+template <typename T, int DIR, bool DST_SMEM, bool ST, bool ODD, int PW = 1, int SH = 4, class Src, class Dst>
 __device__ __forceinline__ void reg_fft(cplx<T>* buf, const FftPlan& fp, int lb, const cplx<T>* tw, const Src& gsrc,
                                         const Dst& gdst) {
   const ShBuf<T, PW, SH> ssrc{buf, lb}, sdst{buf, lb};
@@ -670,26 +749,26 @@ __device__ __forceinline__ void reg_fft(cplx<T>* buf, const FftPlan& fp, int lb,
   if (S == 1) {
     // in place in HBM as well (the column pass and the inverse row pass overwrite their input)
     if (DST_SMEM) {
-      reg_stage_any<T, DIR, ST>(fp, 0, 1, lb, tw, gsrc, sdst, true);
+      reg_stage_any<T, DIR, ST, ODD>(fp, 0, 1, lb, tw, gsrc, sdst, true);
       __syncthreads();
     } else {
-      reg_stage_any<T, DIR, ST>(fp, 0, 1, lb, tw, gsrc, gdst, true);
+      reg_stage_any<T, DIR, ST, ODD>(fp, 0, 1, lb, tw, gsrc, gdst, true);
     }
     return;
   }
-  reg_stage_any<T, DIR, ST>(fp, 0, 1, lb, tw, gsrc, sdst, true);
+  reg_stage_any<T, DIR, ST, ODD>(fp, 0, 1, lb, tw, gsrc, sdst, true);
   __syncthreads();
   int Ns = fp.radix[0];
   for (int s = 1; s < S - 1; ++s) {
-    reg_stage_any<T, DIR, ST>(fp, s, Ns, lb, tw, ssrc, sdst, true);
+    reg_stage_any<T, DIR, ST, ODD>(fp, s, Ns, lb, tw, ssrc, sdst, true);
     __syncthreads();
     Ns *= fp.radix[s];
   }
   if (DST_SMEM) {
-    reg_stage_any<T, DIR, ST>(fp, S - 1, Ns, lb, tw, ssrc, sdst, true);
+    reg_stage_any<T, DIR, ST, ODD>(fp, S - 1, Ns, lb, tw, ssrc, sdst, true);
     __syncthreads();
   } else {
-    reg_stage_any<T, DIR, ST>(fp, S - 1, Ns, lb, tw, ssrc, gdst, false);
+    reg_stage_any<T, DIR, ST, ODD>(fp, S - 1, Ns, lb, tw, ssrc, gdst, false);
   }
 }
 
@@ -701,11 +780,11 @@ constexpr int kRegMaxThreads = 512;
 template <typename T, int DIR, class Src>
 __device__ __forceinline__ void reg_fft_head(cplx<T>* buf, const FftPlan& fp, const cplx<T>* tw, const Src& gsrc) {
   const ShBuf<T, 1> sb{buf, 0};
-  reg_stage_any<T, DIR, false>(fp, 0, 1, 0, tw, gsrc, sb, true);
+  reg_stage_any<T, DIR, false, true>(fp, 0, 1, 0, tw, gsrc, sb, true);
   __syncthreads();
   int Ns = fp.radix[0];
   for (int s = 1; s < fp.nstages - 1; ++s) {
-    reg_stage_any<T, DIR, false>(fp, s, Ns, 0, tw, sb, sb, true);
+    reg_stage_any<T, DIR, false, true>(fp, s, Ns, 0, tw, sb, sb, true);
     __syncthreads();
     Ns *= fp.radix[s];
   }
@@ -762,6 +841,9 @@ __device__ __forceinline__ void r2c_last_split_any(const cplx<T>* buf, const Fft
                                                    cplx<T>* c0, cplx<T>* c1, bool has1) {
   switch (fp.radix[fp.nstages - 1]) {
     case 16: r2c_last_split<T, 16>(buf, fp, tw, c0, c1, has1); break;
+    case 14: r2c_last_split<T, 14>(buf, fp, tw, c0, c1, has1); break;
+    case 10: r2c_last_split<T, 10>(buf, fp, tw, c0, c1, has1); break;
+    case 6: r2c_last_split<T, 6>(buf, fp, tw, c0, c1, has1); break;
     case 12: r2c_last_split<T, 12>(buf, fp, tw, c0, c1, has1); break;
     case 8: r2c_last_split<T, 8>(buf, fp, tw, c0, c1, has1); break;
     case 4: r2c_last_split<T, 4>(buf, fp, tw, c0, c1, has1); break;
@@ -803,7 +885,7 @@ __global__ void DPS_REG_FFT_BOUNDS row_r2c_reg_kernel(Geometry g, FftPlan fp, co
       r2c_last_split_any<T>(buf, fp, tw, c0, c1, has1);
       continue;
     }
-    reg_fft<T, -1, true, false>(buf, fp, 0, tw, src, [](int, int, cplx<T>) {});
+    reg_fft<T, -1, true, false, true>(buf, fp, 0, tw, src, [](int, int, cplx<T>) {});
     for (int k = threadIdx.x; k <= nx / 2; k += blockDim.x) {
       const cplx<T> zk = buf[pad16(k)];
       const cplx<T> zm = conjg(buf[pad16(k == 0 ? 0 : nx - k)]);
@@ -872,6 +954,9 @@ __device__ __forceinline__ void c2r_first_pair_any(cplx<T>* buf, const FftPlan& 
                                                    const cplx<T>* c1, bool has1) {
   switch (fp.radix[0]) {
     case 16: c2r_first_pair<T, 16>(buf, fp, c0, c1, has1); break;
+    case 14: c2r_first_pair<T, 14>(buf, fp, c0, c1, has1); break;
+    case 10: c2r_first_pair<T, 10>(buf, fp, c0, c1, has1); break;
+    case 6: c2r_first_pair<T, 6>(buf, fp, c0, c1, has1); break;
     case 12: c2r_first_pair<T, 12>(buf, fp, c0, c1, has1); break;
     case 8: c2r_first_pair<T, 8>(buf, fp, c0, c1, has1); break;
     case 4: c2r_first_pair<T, 4>(buf, fp, c0, c1, has1); break;
@@ -893,11 +978,11 @@ __device__ __forceinline__ void reg_fft_tail(cplx<T>* buf, const FftPlan& fp, co
   const ShBuf<T, 1> sb{buf, 0};
   int Ns = fp.radix[0];
   for (int s = 1; s < fp.nstages - 1; ++s) {
-    reg_stage_any<T, DIR, false>(fp, s, Ns, 0, tw, sb, sb, true);
+    reg_stage_any<T, DIR, false, true>(fp, s, Ns, 0, tw, sb, sb, true);
     __syncthreads();
     Ns *= fp.radix[s];
   }
-  reg_stage_any<T, DIR, false>(fp, fp.nstages - 1, Ns, 0, tw, sb, gdst, false);
+  reg_stage_any<T, DIR, false, true>(fp, fp.nstages - 1, Ns, 0, tw, sb, gdst, false);
 }
 
 // Row pass, inverse, register-staged: z_k = X0_k + i X1_k over the Hermitian extension, one FFT
@@ -927,7 +1012,7 @@ __global__ void DPS_REG_FFT_BOUNDS row_c2r_reg_kernel(Geometry g, FftPlan fp, co
       });
       continue;
     }
-    reg_fft<T, +1, false, false>(
+    reg_fft<T, +1, false, false, true>(
         buf, fp, 0, tw,
         [&](int e, int) {
           const bool lo = e <= nx / 2;
@@ -944,7 +1029,7 @@ __global__ void DPS_REG_FFT_BOUNDS row_c2r_reg_kernel(Geometry g, FftPlan fp, co
 }
 
 // Column pass, register-staged: cw = 2^lcw adjacent x-wavenumber columns of one plane, along y.
-template <typename T, int DIR>
+template <typename T, int DIR, bool ODD>
 __global__ void DPS_REG_FFT_BOUNDS col_reg_kernel(Geometry g, FftPlan fp, const cplx<T>* __restrict__ tw,
                                                   cplx<T>* __restrict__ grid, const int* __restrict__ zrange, int lcw,
                                                   int kxs, int kxe) {
@@ -958,7 +1043,7 @@ __global__ void DPS_REG_FFT_BOUNDS col_reg_kernel(Geometry g, FftPlan fp, const 
     const int kx0 = kxs + (j << lcw);
     const int ncols = min(cw, kxe - kx0);
     cplx<T>* base = grid + (size_t)(f * g.nz + c) * g.ny * g.pitch + kx0;
-    reg_fft<T, DIR, false, true>(
+    reg_fft<T, DIR, false, true, ODD>(
         buf, fp, lcw, tw,
         [&](int y, int b) { return b < ncols ? base[(size_t)y * g.pitch + b] : mk<T>((T)0, (T)0); },
         [&](int y, int b, cplx<T> v) {
@@ -980,7 +1065,7 @@ template <typename T>
 __host__ __device__ constexpr int pipe_pad_shift() { return sizeof(cplx<T>) == 8 ? 5 : 4; }
 constexpr int kPipeMaxThreadsF = 1024, kPipeMaxThreadsD = 512;
 
-template <typename T, int DIR>
+template <typename T, int DIR, bool ODD>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? kPipeMaxThreadsF : kPipeMaxThreadsD, 1)
     col_pipe_kernel(Geometry g, FftPlan fp, const cplx<T>* __restrict__ tw, cplx<T>* __restrict__ grid,
                     const int* __restrict__ zrange, int lcw, int kxs, int kxe) {
@@ -1030,7 +1115,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kPipeMaxThreadsF : kPipeMaxTh
     cp_wait_all();
     __syncthreads();  // this unit staged; every thread is done with the previous unit (in nxt)
     if (u + gridDim.x < um.total) issue(u + gridDim.x, nxt);
-    reg_fft<T, DIR, false, true, PW, SH>(
+    reg_fft<T, DIR, false, true, ODD, PW, SH>(
         cur, fp, lcw, tw,
         ShBuf<T, PW, SH>{cur, lcw},
         [&](int y, int b, cplx<T> v) {
@@ -1085,7 +1170,7 @@ __host__ __device__ __forceinline__ int tma_buf_len(int points) {
   return (n + q - 1) / q * q;
 }
 
-template <typename T, int DIR>
+template <typename T, int DIR, bool ODD>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? kPipeMaxThreadsF : kPipeMaxThreadsD, 1)
     col_tma_kernel(const __grid_constant__ CUtensorMap tmap, Geometry g, FftPlan fp, const cplx<T>* __restrict__ tw,
                    cplx<T>* __restrict__ grid, const int* __restrict__ zrange, int* __restrict__ status, int lcw,
@@ -1139,7 +1224,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kPipeMaxThreadsF : kPipeMaxTh
     const int kx0 = kxs + (j << lcw);
     const int ncols = min(cw, kxe - kx0);
     cplx<T>* base = grid + (size_t)(f * g.nz + c) * g.ny * g.pitch + kx0;
-    reg_fft<T, DIR, false, true, PW, SH>(cur, fp, lcw, tw, ShBuf<T, 0, SH>{cur, lcw},
+    reg_fft<T, DIR, false, true, ODD, PW, SH>(cur, fp, lcw, tw, ShBuf<T, 0, SH>{cur, lcw},
                                          [&](int y, int b, cplx<T> v) {
                                            if (b < ncols) base[(size_t)y * g.pitch + b] = v;
                                          });
@@ -1169,11 +1254,12 @@ constexpr int kFftMaxThreads = 512;
 // threads for a transform of `points` values: at most kFftPer per thread, whole warps
 int fft_threads(int points) { return std::max(32, (points + kFftPer * 32 - 1) / (kFftPer * 32) * 32); }
 
-// log2 of the column block: the widest (at most 8 columns) within the thread limit whose staging,
-// work and twiddle buffers fit in 190 KB of shared memory
+// log2 of the column block: the widest within the thread limit whose staging, work and twiddle buffers fit
+// in 190 KB of shared memory; at most 8 columns in float, 4 in double (a 64-byte row piece either way;
+// double at 384 rows: 2.16 ms at 8 columns, 1.96 at 4, 2.26 at 2)
 template <typename T>
 int col_lwidth(const Plan& p) {
-  for (int l = 3; l > 0; --l)
+  for (int l = sizeof(T) == 4 ? 3 : 2; l > 0; --l)
     if (fft_threads(p.g.ny << l) <= kFftMaxThreads && col_smem<T>(p.g, l) <= 190 * 1024) return l;
   return 0;
 }
@@ -1203,8 +1289,6 @@ template <typename T>
 bool reg_fits(const FftPlan& fp, int lb) {
   return reg_threads(fp, lb) <= kRegMaxThreads && reg_smem<T>(fp.n << lb) <= 100 * 1024;
 }
-
-}  // namespace
 
 template <typename T>
 size_t pipe_smem(int points) {
@@ -1251,211 +1335,6 @@ bool encode_col_tmap(Plan& p, int lcw, int bh) {
                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <typename T>
-int fft_set_col_width(Plan& p, int lcw, int reg) {
-  if (lcw < 0 || lcw > 3 || reg < 0 || reg > 3) return 0;
-  if (reg == 3) {
-    const int maxth = sizeof(T) == 4 ? kPipeMaxThreadsF : kPipeMaxThreadsD;
-    const int th = reg_threads(p.fyr, lcw);
-    const size_t sm = tma_smem<T>(p.g.ny << lcw);
-    const int bh = tma_box_rows<T>(p.g.ny, lcw);
-    // box rows of 16-byte multiples; a block never reads past the padded row (pitch is a multiple
-    // of 32 columns and a block starts at a multiple of its width)
-    if (th > maxth || sm > 224 * 1024 || bh == 0 || ((2u << lcw) * sizeof(T)) % 16 != 0) return 0;
-    if (!encode_col_tmap<T>(p, lcw, bh)) return 0;
-    p.col_lcw = lcw;
-    p.fft_reg[1] = 3;
-    p.col_tma_rows = bh;
-    p.fft_grid[2] = resident_grid(col_tma_kernel<T, -1>, th, sm, p.device);
-    p.fft_grid[3] = resident_grid(col_tma_kernel<T, +1>, th, sm, p.device);
-    return 1;
-  }
-  if (reg == 2) {
-    if (!pipe_fits<T>(p.fyr, lcw)) return 0;
-    const int th = reg_threads(p.fyr, lcw);
-    const size_t sm = pipe_smem<T>(p.g.ny << lcw);
-    p.col_lcw = lcw;
-    p.fft_reg[1] = 2;
-    p.fft_grid[2] = resident_grid(col_pipe_kernel<T, -1>, th, sm, p.device);
-    p.fft_grid[3] = resident_grid(col_pipe_kernel<T, +1>, th, sm, p.device);
-    return 1;
-  }
-  if (reg) {
-    if (!reg_fits<T>(p.fyr, lcw)) return 0;
-    const int th = reg_threads(p.fyr, lcw);
-    const size_t sm = reg_smem<T>(p.g.ny << lcw);
-    p.col_lcw = lcw;
-    p.fft_reg[1] = 1;
-    p.fft_grid[2] = resident_grid(col_reg_kernel<T, -1>, th, sm, p.device);
-    p.fft_grid[3] = resident_grid(col_reg_kernel<T, +1>, th, sm, p.device);
-    return 1;
-  }
-  const size_t col = col_smem<T>(p.g, lcw);
-  const int tcol = fft_threads(p.g.ny << lcw);
-  if (tcol > kFftMaxThreads || col > 220 * 1024) return 0;
-  p.col_lcw = lcw;
-  p.fft_reg[1] = 0;
-  p.fft_grid[2] = resident_grid(col_kernel<T, -1>, tcol, col, p.device);
-  p.fft_grid[3] = resident_grid(col_kernel<T, +1>, tcol, col, p.device);
-  return 1;
-}
-
-template <typename T>
-int fft_set_row_variant(Plan& p, int reg) {
-  if (reg) {
-    if (!reg_fits<T>(p.fxr, 0)) return 0;
-    const int th = reg_threads(p.fxr, 0);
-    const size_t sm = reg_smem<T>(p.g.nx);
-    p.fft_reg[0] = 1;
-    p.fft_grid[0] = r2c_split_ok(p.fxr) ? resident_grid(row_r2c_reg_kernel<T, true>, th, sm, p.device)
-                                         : resident_grid(row_r2c_reg_kernel<T, false>, th, sm, p.device);
-    p.fft_grid[1] = c2r_pair_ok(p.fxr) ? resident_grid(row_c2r_reg_kernel<T, true>, th, sm, p.device)
-                                        : resident_grid(row_c2r_reg_kernel<T, false>, th, sm, p.device);
-    return 1;
-  }
-  const size_t r2c = row_r2c_smem<T>(p.g), c2r = row_c2r_smem<T>(p.g);
-  const int trow = fft_threads(p.g.nx);
-  if (trow > kFftMaxThreads || r2c > 220 * 1024 || c2r > 220 * 1024) return 0;
-  p.fft_reg[0] = 0;
-  p.fft_grid[0] = resident_grid(row_r2c_kernel<T>, trow, r2c, p.device);
-  p.fft_grid[1] = resident_grid(row_c2r_kernel<T>, trow, c2r, p.device);
-  return 1;
-}
-
-// Default shapes, from measurements on rollers and slit grids (3072^2, 768^2, 384^2): the
-// register-staged row pass only for long float rows whose stages keep at least 3/4 of the block
-// busy (3072 = 16 x 16 x 12: 10 % faster than the shared-memory-staged pass; 768 = 16 x 16 x 3 and
-// 384 = 16 x 12 x 2 leave most threads idle in the radix-16 stages and run 1.5-2.5x slower, as does
-// FP64).  Columns: the width of a block's per-row piece decides (3072 rows, mixed: 2 columns
-// shared-memory-staged 18.1 ms per pass pair, 4 columns prefetched register-staged 14.5 ms, the
-// latter at 2 columns 23.6 ms), so the prefetched register-staged pass where its two buffers fit a
-// wider block than the staged pass's three, else the staged pass at its widest; the register-staged
-// pass without prefetch (loads exposed; 1.3-1.5x slower at equal width) only by hand or autotuning.
-template <typename T>
-bool reg_rows_default(const FftPlan& fp) {
-  if (sizeof(T) != 4 || fp.n < 2048 || !reg_fits<T>(fp, 0)) return false;
-  int rmin = fp.radix[0], rmax = fp.radix[0];
-  for (int s = 1; s < fp.nstages; ++s) {
-    rmin = std::min(rmin, fp.radix[s]);
-    rmax = std::max(rmax, fp.radix[s]);
-  }
-  return 3 * rmax <= 4 * rmin;
-}
-
-template <typename T>
-int fft_smem_ok(Plan& p) {
-  if (!allow_smem(row_r2c_kernel<T>) || !allow_smem(row_c2r_kernel<T>) || !allow_smem(col_kernel<T, -1>) ||
-      !allow_smem(col_kernel<T, +1>) || !allow_smem(row_r2c_reg_kernel<T, false>) ||
-      !allow_smem(row_r2c_reg_kernel<T, true>) || !allow_smem(row_c2r_reg_kernel<T, false>) ||
-      !allow_smem(row_c2r_reg_kernel<T, true>) ||
-      !allow_smem(col_reg_kernel<T, -1>) || !allow_smem(col_reg_kernel<T, +1>) ||
-      !allow_smem(col_pipe_kernel<T, -1>) || !allow_smem(col_pipe_kernel<T, +1>) ||
-      !allow_smem(col_tma_kernel<T, -1>) || !allow_smem(col_tma_kernel<T, +1>))
-    return 0;
-  const bool rr = reg_rows_default<T>(p.fxr);
-  if (!fft_set_row_variant<T>(p, rr ? 1 : 0) && !fft_set_row_variant<T>(p, rr ? 0 : 1)) return 0;
-  // columns: the prefetched register-staged pass when it fits a wider block than the staged one,
-  // prefetched by TMA where a box shape fits (3072^2: 12.2 -> 10.7 ms per pass pair), else cp.async
-  const int ls = col_lwidth<T>(p);
-  for (int l = 3; l > ls; --l)
-    if (fft_set_col_width<T>(p, l, 3) || fft_set_col_width<T>(p, l, 2)) return 1;
-  // at the staged pass's width, TMA on long columns (768 rows, 8 columns: 0.78 -> 0.70 ms per pass
-  // pair; 384 rows: 0.57 staged against 0.66, the units too short for the per-unit barrier work)
-  if (p.g.ny >= 512 && fft_set_col_width<T>(p, ls, 3)) return 1;
-  if (fft_set_col_width<T>(p, ls, 0)) return 1;
-  for (int l = 3; l >= 0; --l)
-    if (fft_set_col_width<T>(p, l, 1)) return 1;
-  return 0;
-}
-
-template <typename T>
-void launch_fft_rows(const Plan& p, int dir, cudaStream_t s) {
-  const Geometry& g = p.g;
-  const cplx<T>* twx = reinterpret_cast<const cplx<T>*>(p.tab.twx);
-  if (p.fft_reg[0]) {
-    const int th = reg_threads(p.fxr, 0);
-    const size_t sm = reg_smem<T>(g.nx);
-    T* grid = reinterpret_cast<T*>(p.grid);
-    if (dir < 0 && r2c_split_ok(p.fxr))
-      row_r2c_reg_kernel<T, true><<<p.fft_grid[0], th, sm, s>>>(g, p.fxr, twx, grid, p.zrange);
-    else if (dir < 0)
-      row_r2c_reg_kernel<T, false><<<p.fft_grid[0], th, sm, s>>>(g, p.fxr, twx, grid, p.zrange);
-    else if (c2r_pair_ok(p.fxr))
-      row_c2r_reg_kernel<T, true><<<p.fft_grid[1], th, sm, s>>>(g, p.fxr, twx, grid, p.zrange);
-    else
-      row_c2r_reg_kernel<T, false><<<p.fft_grid[1], th, sm, s>>>(g, p.fxr, twx, grid, p.zrange);
-    return;
-  }
-  const int th = fft_threads(g.nx);
-  if (dir < 0)
-    row_r2c_kernel<T><<<p.fft_grid[0], th, row_r2c_smem<T>(g), s>>>(g, p.fx, twx, reinterpret_cast<T*>(p.grid),
-                                                                      p.zrange);
-  else
-    row_c2r_kernel<T><<<p.fft_grid[1], th, row_c2r_smem<T>(g), s>>>(g, p.fx, twx, reinterpret_cast<T*>(p.grid),
-                                                                      p.zrange);
-}
-
-template <typename T>
-void launch_fft_cols(const Plan& p, int dir, int kxs, int kxe, cudaStream_t s) {
-  const Geometry& g = p.g;
-  const cplx<T>* twy = reinterpret_cast<const cplx<T>*>(p.tab.twy);
-  const int lcw = p.col_lcw;
-  cplx<T>* grid = reinterpret_cast<cplx<T>*>(p.grid);
-  const cplx<T>* tsy = reinterpret_cast<const cplx<T>*>(p.tab.tsy);
-  if (p.fft_reg[1] == 3) {
-    const int th = reg_threads(p.fyr, lcw);
-    const size_t sm = tma_smem<T>(g.ny << lcw);
-    const CUtensorMap& map = *reinterpret_cast<const CUtensorMap*>(p.col_tmap);
-    if (dir < 0)
-      col_tma_kernel<T, -1><<<p.fft_grid[2], th, sm, s>>>(map, g, p.fyr, tsy, grid, p.zrange, p.status, lcw, kxs, kxe,
-                                                          p.col_tma_rows, p.inject == 3 ? 1 : 0);
-    else
-      col_tma_kernel<T, +1><<<p.fft_grid[3], th, sm, s>>>(map, g, p.fyr, tsy, grid, p.zrange, p.status, lcw, kxs, kxe,
-                                                          p.col_tma_rows, 0);
-    return;
-  }
-  if (p.fft_reg[1] == 2) {
-    const int th = reg_threads(p.fyr, lcw);
-    const size_t sm = pipe_smem<T>(g.ny << lcw);
-    if (dir < 0)
-      col_pipe_kernel<T, -1><<<p.fft_grid[2], th, sm, s>>>(g, p.fyr, tsy, grid, p.zrange, lcw, kxs, kxe);
-    else
-      col_pipe_kernel<T, +1><<<p.fft_grid[3], th, sm, s>>>(g, p.fyr, tsy, grid, p.zrange, lcw, kxs, kxe);
-    return;
-  }
-  if (p.fft_reg[1]) {
-    const int th = reg_threads(p.fyr, lcw);
-    const size_t sm = reg_smem<T>(g.ny << lcw);
-    if (dir < 0)
-      col_reg_kernel<T, -1><<<p.fft_grid[2], th, sm, s>>>(g, p.fyr, tsy, grid, p.zrange, lcw, kxs, kxe);
-    else
-      col_reg_kernel<T, +1><<<p.fft_grid[3], th, sm, s>>>(g, p.fyr, tsy, grid, p.zrange, lcw, kxs, kxe);
-    return;
-  }
-  const size_t sm = col_smem<T>(g, lcw);
-  const int th = fft_threads(g.ny << lcw);
-  if (dir < 0)
-    col_kernel<T, -1><<<p.fft_grid[2], th, sm, s>>>(g, p.fy, twy, reinterpret_cast<cplx<T>*>(p.grid), p.zrange, lcw,
-                                                    kxs, kxe);
-  else
-    col_kernel<T, +1><<<p.fft_grid[3], th, sm, s>>>(g, p.fy, twy, reinterpret_cast<cplx<T>*>(p.grid), p.zrange, lcw,
-                                                    kxs, kxe);
-}
-
-template int fft_smem_ok<float>(Plan&);
-template int fft_smem_ok<double>(Plan&);
-template int fft_set_row_variant<float>(Plan&, int);
-template int fft_set_row_variant<double>(Plan&, int);
-template int fft_set_col_width<float>(Plan&, int, int);
-template int fft_set_col_width<double>(Plan&, int, int);
-template void launch_fft_rows<float>(const Plan&, int, cudaStream_t);
-template void launch_fft_rows<double>(const Plan&, int, cudaStream_t);
-template void launch_fft_cols<float>(const Plan&, int, int, int, cudaStream_t);
-template void launch_fft_cols<double>(const Plan&, int, int, int, cudaStream_t);
-
-template <typename T>
-int fft_col_width(const Plan& p) { return 1 << p.col_lcw; }
-template int fft_col_width<float>(const Plan&);
-template int fft_col_width<double>(const Plan&);
+}  // namespace
 
 }  // namespace dps

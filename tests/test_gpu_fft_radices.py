@@ -1,0 +1,37 @@
+"""Every radix of the xy transforms (2 to 16, composite ones among them) in every pass variant that fits,
+against the oracle at the parity bars: 210 = 15 x 14, 90 = 10 x 9, 126 = 14 x 9, 225 = 15 x 15, 150 = 15 x 10,
+36 = 6 x 6, 98 = 14 x 7, 96 = 12 x 8."""
+
+import pytest
+
+from gpu_helpers import gpu_mobility, oracle_params, rel_l2, small_params
+from oracle.stokes import mobility
+from paper_2210_01837_gb300 import binding
+from paper_2210_01837_gb300.workloads import random_particles
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp64": 1e-9, "mixed": 1e-5}
+
+
+@pytest.mark.parametrize("nx,ny", [(210, 36), (36, 210), (126, 90), (90, 126), (150, 98), (96, 225)])
+def test_every_radix_in_every_variant_matches_oracle(nx, ny):
+    params = small_params("bottom_wall", nx=nx, ny=ny, nz=13, zmax=4.0, torque=True)
+    pos, F, T = random_particles(params, 12, seed=nx + ny)
+    U_ref, W_ref = mobility(oracle_params(params), pos, F, T)
+    for precision in ("fp64", "mixed"):
+        plan = binding.Plan.from_params(params, with_torque=True, precision=precision, max_n=len(pos))
+        tried = 0
+        for rows in (0, 1):
+            for cols in (0, 1, 2, 3):
+                for width in (1, 2, 4, 8):
+                    try:
+                        plan.set_fft(rows, cols, width)
+                    except binding.DpsError:
+                        continue  # the shape does not fit
+                    tried += 1
+                    U, W = gpu_mobility(params, pos, F, T, precision, plan=plan)
+                    assert rel_l2(U, U_ref) <= TOL[precision], (precision, rows, cols, width)
+                    assert rel_l2(W, W_ref) <= TOL[precision], (precision, rows, cols, width)
+        assert tried >= 8
+        plan.close()
