@@ -438,29 +438,35 @@ void enqueue(Plan& p, int64_t n, const double* pos, const double* F, const doubl
     launch_fft_cols<T>(p, -1, 0, p.g.nkx, s);
     return;
   }
-  // wavenumber space, column chunks: y-FFT + Chebyshev forward on s, FP64 solve on side[0],
-  // backward + inverse y-FFT on side[1]; the FP64-bound solve of one chunk overlaps the float and
-  // memory-bound work of its neighbours
-  cudaStream_t ss = p.side[0], sb = p.side[1];
-  cudaEventRecord(p.ev_fork, s);
-  cudaStreamWaitEvent(ss, p.ev_fork, 0);
-  cudaStreamWaitEvent(sb, p.ev_fork, 0);
   const bool inverse = last_stage >= 5;
-  for (int j = 0; j < p.nchunks; ++j) {
-    const int x0 = p.chunk_x0[j], x1 = p.chunk_x0[j + 1];
-    timed(5, s, [&] { launch_fft_cols<T>(p, -1, x0, x1, s); });
-    timed(6, s, [&] { launch_bvp<T>(p, 0, x0, x1 - x0, s); });
-    cudaEventRecord(p.ev_f[j], s);
-    cudaStreamWaitEvent(ss, p.ev_f[j], 0);
-    timed(7, ss, [&] { launch_bvp<T>(p, 1, x0, x1 - x0, ss); });
-    cudaEventRecord(p.ev_s[j], ss);
-    cudaStreamWaitEvent(sb, p.ev_s[j], 0);
-    timed(8, sb, [&] { launch_bvp<T>(p, 2, x0, x1 - x0, sb); });
-    if (inverse) timed(9, sb, [&] { launch_fft_cols<T>(p, +1, x0, x1, sb); });
-    cudaEventRecord(p.ev_b[j], sb);
+  if (p.nchunks == 1) {  // one chunk: everything in the caller's stream, no events between the stages
+    timed(5, s, [&] { launch_fft_cols<T>(p, -1, 0, p.g.nkx, s); });
+    for (int part = 0; part < 3; ++part) timed(6 + part, s, [&] { launch_bvp<T>(p, part, 0, p.g.nkx, s); });
+    if (inverse) timed(9, s, [&] { launch_fft_cols<T>(p, +1, 0, p.g.nkx, s); });
+  } else {
+    // wavenumber space, column chunks: y-FFT + Chebyshev forward on s, FP64 solve on side[0],
+    // backward + inverse y-FFT on side[1]; the FP64-bound solve of one chunk overlaps the float and
+    // memory-bound work of its neighbours
+    cudaStream_t ss = p.side[0], sb = p.side[1];
+    cudaEventRecord(p.ev_fork, s);
+    cudaStreamWaitEvent(ss, p.ev_fork, 0);
+    cudaStreamWaitEvent(sb, p.ev_fork, 0);
+    for (int j = 0; j < p.nchunks; ++j) {
+      const int x0 = p.chunk_x0[j], x1 = p.chunk_x0[j + 1];
+      timed(5, s, [&] { launch_fft_cols<T>(p, -1, x0, x1, s); });
+      timed(6, s, [&] { launch_bvp<T>(p, 0, x0, x1 - x0, s); });
+      cudaEventRecord(p.ev_f[j], s);
+      cudaStreamWaitEvent(ss, p.ev_f[j], 0);
+      timed(7, ss, [&] { launch_bvp<T>(p, 1, x0, x1 - x0, ss); });
+      cudaEventRecord(p.ev_s[j], ss);
+      cudaStreamWaitEvent(sb, p.ev_s[j], 0);
+      timed(8, sb, [&] { launch_bvp<T>(p, 2, x0, x1 - x0, sb); });
+      if (inverse) timed(9, sb, [&] { launch_fft_cols<T>(p, +1, x0, x1, sb); });
+      cudaEventRecord(p.ev_b[j], sb);
+    }
+    cudaStreamWaitEvent(s, p.ev_b[p.nchunks - 1], 0);
+    cudaStreamWaitEvent(s, p.ev_s[p.nchunks - 1], 0);
   }
-  cudaStreamWaitEvent(s, p.ev_b[p.nchunks - 1], 0);
-  cudaStreamWaitEvent(s, p.ev_s[p.nchunks - 1], 0);
   if (!inverse) return;
   timed(10, s, [&] { launch_fft_rows<T>(p, +1, s); });
   if (last_stage <= 5) return;
