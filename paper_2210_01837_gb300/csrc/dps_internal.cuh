@@ -151,6 +151,7 @@ struct Plan {
   int bvp_blocks;       // persistent grid size of the per-k solver
   int fft_grid[4];      // resident grids of the persistent FFT passes: rows fwd/inv, columns fwd/inv
   int col_lcw;          // log2 of the column block of the y-FFT pass (default rule or autotuned)
+  int row_lb;           // log2 of the row pairs per block of the staged row passes
   int fft_reg[2];       // FFT variant of the row and the column pass: 0 smem-staged, 1 register-staged,
                         // 2 (columns) register-staged with cp.async prefetch, 3 (columns) the same with
                         // TMA box loads

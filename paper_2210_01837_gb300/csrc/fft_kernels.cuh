@@ -414,109 +414,138 @@ struct UnitMap {
   }
 };
 
+// The half-spectrum split of two packed real rows: X0_k = (z_k + conj z_{n-k}) / 2 and
+// X1_k = (z_k - conj z_{n-k}) / (2i), given z_k and zn = z_{n-k}.
+template <typename T>
+__device__ __forceinline__ void split_store(cplx<T>* c0, cplx<T>* c1, bool has1, int k, cplx<T> zk, cplx<T> zn) {
+  const T half = (T)0.5;
+  const cplx<T> zm = conjg(zn);
+  c0[k] = scl(zk + zm, half);
+  if (has1) {
+    const cplx<T> d = zk - zm;
+    c1[k] = mk<T>(half * d.y, -half * d.x);
+  }
+}
+
 // real rows rounded up so that the second staged row stays 16-byte aligned
 __host__ __device__ __forceinline__ int staged_len(int n) { return (n + 3) & ~3; }
 
-// Row pass, forward: a unit is two real rows y0 = 2j, y1 = 2j + 1, packed as z = r0 + i r1.
-template <typename T>
+// Row pass, forward: a unit is 2^lb pairs of real rows, each pair packed as z = r0 + i r1; the pairs are
+// interleaved sequences, so that a short row's few butterflies fill whole warps.
+template <typename T, bool MULTI>
 __global__ void __launch_bounds__(512, 1) row_r2c_kernel(Geometry g, FftPlan fp, const cplx<T>* __restrict__ tw,
-                                                         T* __restrict__ grid, const int* __restrict__ zrange) {
+                                                         T* __restrict__ grid, const int* __restrict__ zrange, int lb_arg) {
+  const int lb = MULTI ? lb_arg : 0;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int nx = g.nx, nxr = staged_len(nx);
-  T* raw = reinterpret_cast<T*>(smraw);  // [2][nxr] staged rows
-  cplx<T>* b0 = reinterpret_cast<cplx<T>*>(raw + 2 * nxr);
-  cplx<T>* b1 = b0 + pad16(nx) + 1;
-  cplx<T>* stw = b1 + pad16(nx) + 1;  // twiddle table, staged once per (persistent) block
+  const int nx = g.nx, nxr = staged_len(nx), nr = 2 << lb;
+  T* raw = reinterpret_cast<T*>(smraw);  // [nr][nxr] staged rows
+  cplx<T>* b0 = reinterpret_cast<cplx<T>*>(raw + nr * nxr);
+  cplx<T>* b1 = b0 + pad16(nx << lb) + 1;
+  cplx<T>* stw = b1 + pad16(nx << lb) + 1;  // twiddle table, staged once per (persistent) block
   for (int i = threadIdx.x; i < nx; i += blockDim.x) stw[i] = tw[i];
-  const UnitMap um(g, zrange, (g.ny + 1) / 2);
+  const UnitMap um(g, zrange, (g.ny + nr - 1) >> (lb + 1));
   const size_t rowlen = (size_t)2 * g.pitch;
-  auto row0_of = [&](long long u, bool& has1) {
+  auto row0_of = [&](long long u, int& have) {
     int f, c, j;
     um.at(u, f, c, j);
-    has1 = 2 * j + 1 < g.ny;
-    return grid + ((size_t)(f * g.nz + c) * g.ny + 2 * j) * rowlen;
+    have = min(nr, g.ny - nr * j);
+    return grid + ((size_t)(f * g.nz + c) * g.ny + nr * j) * rowlen;
   };
   auto issue = [&](long long u) {
-    bool has1;
-    const T* r0 = row0_of(u, has1);
+    int have;
+    const T* r0 = row0_of(u, have);
     async_bytes(raw, r0, nx * (int)sizeof(T));
-    if (has1) async_bytes(raw + nxr, r0 + rowlen, nx * (int)sizeof(T));
+    if (!MULTI && have > 1) async_bytes(raw + nxr, r0 + rowlen, nx * (int)sizeof(T));
+    if (MULTI)
+      for (int r = 1; r < have; ++r) async_bytes(raw + r * nxr, r0 + r * rowlen, nx * (int)sizeof(T));
     cp_commit();
+    if (have & 1)  // the last row's missing partner; pairs wholly absent transform what is there, unread
+      for (int i = threadIdx.x; i < nx; i += blockDim.x) raw[have * nxr + i] = (T)0;
   };
+  // epilogue: consecutive threads take consecutive wavenumbers of one pair
+  const int per = (int)blockDim.x >> lb, eb = MULTI ? (int)threadIdx.x / per : 0, ek = (int)threadIdx.x - eb * per;
   long long u = blockIdx.x;
   if (u < um.total) issue(u);
   for (; u < um.total; u += gridDim.x) {
-    bool has1;
-    T* row0 = row0_of(u, has1);
+    int have;
+    T* row0 = row0_of(u, have);
     cp_wait_all();
     __syncthreads();  // staged rows visible; the previous unit's epilogue is done with buf
-    fft_first<T, -1>(b0, fp, 0, [&](int e) { return mk<T>(raw[e], has1 ? raw[nxr + e] : (T)0); });
+    fft_first<T, -1>(b0, fp, lb, [&](int i) {
+      const int e = i >> lb, r = 2 * (i & ((1 << lb) - 1));
+      return mk<T>(raw[r * nxr + e], raw[(r + 1) * nxr + e]);
+    });
     __syncthreads();  // staging buffer consumed
     if (u + gridDim.x < um.total) issue(u + gridDim.x);
-    const cplx<T>* buf = fft_rest<T, -1>(b0, b1, fp, 0, stw);
-    cplx<T>* c0 = reinterpret_cast<cplx<T>*>(row0);
-    cplx<T>* c1 = reinterpret_cast<cplx<T>*>(row0 + rowlen);
-    const T half = (T)0.5;
-    for (int k = threadIdx.x; k <= nx / 2; k += blockDim.x) {
-      const cplx<T> zk = buf[pad16(k)];
-      const cplx<T> zm = conjg(buf[pad16(k == 0 ? 0 : nx - k)]);
-      c0[k] = scl(zk + zm, half);
-      if (has1) {
-        const cplx<T> d = zk - zm;  // (zk - conj z_{-k}) / (2i)
-        c1[k] = mk<T>(half * d.y, -half * d.x);
-      }
+    const cplx<T>* buf = fft_rest<T, -1>(b0, b1, fp, lb, stw);
+    if (!MULTI || 2 * eb < have) {
+      const bool has1 = 2 * eb + 1 < have;
+      cplx<T>* c0 = reinterpret_cast<cplx<T>*>(row0 + 2 * eb * rowlen);
+      cplx<T>* c1 = reinterpret_cast<cplx<T>*>(row0 + (2 * eb + 1) * rowlen);
+      for (int k = ek; k <= nx / 2; k += per)
+        split_store<T>(c0, c1, has1, k, buf[pad16((k << lb) + eb)], buf[pad16(((k == 0 ? 0 : nx - k) << lb) + eb)]);
     }
   }
 }
 
-// Row pass, inverse: two half spectra -> z with z_k = X0_k + i X1_k (Hermitian extension), one FFT.
-template <typename T>
+// Row pass, inverse: 2^lb pairs of half spectra -> z with z_k = X0_k + i X1_k (Hermitian extension), one
+// FFT each.
+template <typename T, bool MULTI>
 __global__ void __launch_bounds__(512, 1) row_c2r_kernel(Geometry g, FftPlan fp, const cplx<T>* __restrict__ tw,
-                                                         T* __restrict__ grid, const int* __restrict__ zrange) {
+                                                         T* __restrict__ grid, const int* __restrict__ zrange, int lb_arg) {
+  const int lb = MULTI ? lb_arg : 0;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int nx = g.nx, nh = nx / 2 + 1, nhr = (nh + 1) & ~1;
-  cplx<T>* raw = reinterpret_cast<cplx<T>*>(smraw);  // [2][nhr] staged half spectra
-  cplx<T>* b0 = raw + 2 * nhr;
-  cplx<T>* b1 = b0 + pad16(nx) + 1;
-  cplx<T>* stw = b1 + pad16(nx) + 1;  // twiddle table, staged once per (persistent) block
+  const int nx = g.nx, nh = nx / 2 + 1, nhr = (nh + 1) & ~1, nr = 2 << lb;
+  cplx<T>* raw = reinterpret_cast<cplx<T>*>(smraw);  // [nr][nhr] staged half spectra
+  cplx<T>* b0 = raw + nr * nhr;
+  cplx<T>* b1 = b0 + pad16(nx << lb) + 1;
+  cplx<T>* stw = b1 + pad16(nx << lb) + 1;  // twiddle table, staged once per (persistent) block
   for (int i = threadIdx.x; i < nx; i += blockDim.x) stw[i] = tw[i];
-  const UnitMap um(g, zrange, (g.ny + 1) / 2);
+  const UnitMap um(g, zrange, (g.ny + nr - 1) >> (lb + 1));
   const size_t rowlen = (size_t)2 * g.pitch;
-  auto row0_of = [&](long long u, bool& has1) {
+  auto row0_of = [&](long long u, int& have) {
     int f, c, j;
     um.at(u, f, c, j);
-    has1 = 2 * j + 1 < g.ny;
-    return grid + ((size_t)(f * g.nz + c) * g.ny + 2 * j) * rowlen;
+    have = min(nr, g.ny - nr * j);
+    return grid + ((size_t)(f * g.nz + c) * g.ny + nr * j) * rowlen;
   };
   auto issue = [&](long long u) {
-    bool has1;
-    const T* r0 = row0_of(u, has1);
+    int have;
+    const T* r0 = row0_of(u, have);
     async_bytes(raw, r0, nh * (int)sizeof(cplx<T>));
-    if (has1) async_bytes(raw + nhr, r0 + rowlen, nh * (int)sizeof(cplx<T>));
+    if (!MULTI && have > 1) async_bytes(raw + nhr, r0 + rowlen, nh * (int)sizeof(cplx<T>));
+    if (MULTI)
+      for (int r = 1; r < have; ++r) async_bytes(raw + r * nhr, r0 + r * rowlen, nh * (int)sizeof(cplx<T>));
     cp_commit();
+    if (have & 1)
+      for (int i = threadIdx.x; i < nh; i += blockDim.x) raw[have * nhr + i] = mk<T>((T)0, (T)0);
   };
+  const int per = (int)blockDim.x >> lb, eb = MULTI ? (int)threadIdx.x / per : 0, ek = (int)threadIdx.x - eb * per;
   long long u = blockIdx.x;
   if (u < um.total) issue(u);
   for (; u < um.total; u += gridDim.x) {
-    bool has1;
-    T* row0 = row0_of(u, has1);
-    T* row1 = row0 + rowlen;
+    int have;
+    T* row0 = row0_of(u, have);
     cp_wait_all();
     __syncthreads();
-    fft_first<T, +1>(b0, fp, 0, [&](int e) {
+    fft_first<T, +1>(b0, fp, lb, [&](int i) {
+      const int e = i >> lb, r = 2 * (i & ((1 << lb) - 1));
       const bool lo = e <= nx / 2;
       const int k = lo ? e : nx - e;
-      const cplx<T> x0 = raw[k];
-      const cplx<T> x1 = has1 ? raw[nhr + k] : mk<T>((T)0, (T)0);
+      const cplx<T> x0 = raw[r * nhr + k], x1 = raw[(r + 1) * nhr + k];
       return lo ? x0 + mul_i(x1) : conjg(x0) + mul_i(conjg(x1));
     });
     __syncthreads();
     if (u + gridDim.x < um.total) issue(u + gridDim.x);
-    const cplx<T>* buf = fft_rest<T, +1>(b0, b1, fp, 0, stw);
-    for (int a = threadIdx.x; a < nx; a += blockDim.x) {
-      const cplx<T> v = buf[pad16(a)];
-      row0[a] = v.x;
-      if (has1) row1[a] = v.y;
+    const cplx<T>* buf = fft_rest<T, +1>(b0, b1, fp, lb, stw);
+    if (!MULTI || 2 * eb < have) {
+      const bool has1 = 2 * eb + 1 < have;
+      T *row = row0 + 2 * eb * rowlen, *row1 = row + rowlen;
+      for (int a = ek; a < nx; a += per) {
+        const cplx<T> v = buf[pad16((a << lb) + eb)];
+        row[a] = v.x;
+        if (has1) row1[a] = v.y;
+      }
     }
   }
 }
@@ -787,19 +816,6 @@ __device__ __forceinline__ void reg_fft_head(cplx<T>* buf, const FftPlan& fp, co
     reg_stage_any<T, DIR, false, true>(fp, s, Ns, 0, tw, sb, sb, true);
     __syncthreads();
     Ns *= fp.radix[s];
-  }
-}
-
-// The half-spectrum split of two packed real rows: X0_k = (z_k + conj z_{n-k}) / 2 and
-// X1_k = (z_k - conj z_{n-k}) / (2i), given z_k and zn = z_{n-k}.
-template <typename T>
-__device__ __forceinline__ void split_store(cplx<T>* c0, cplx<T>* c1, bool has1, int k, cplx<T> zk, cplx<T> zn) {
-  const T half = (T)0.5;
-  const cplx<T> zm = conjg(zn);
-  c0[k] = scl(zk + zm, half);
-  if (has1) {
-    const cplx<T> d = zk - zm;
-    c1[k] = mk<T>(half * d.y, -half * d.x);
   }
 }
 
@@ -1234,13 +1250,13 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kPipeMaxThreadsF : kPipeMaxTh
 size_t padded_bytes(int n, size_t esz) { return (size_t)(n + (n >> 4) + 1) * esz; }
 
 template <typename T>
-size_t row_r2c_smem(const Geometry& g) {
-  return (size_t)2 * staged_len(g.nx) * sizeof(T) + 2 * padded_bytes(g.nx, sizeof(cplx<T>)) +
+size_t row_r2c_smem(const Geometry& g, int lb) {
+  return (size_t)(2 << lb) * staged_len(g.nx) * sizeof(T) + 2 * padded_bytes(g.nx << lb, sizeof(cplx<T>)) +
          (size_t)g.nx * sizeof(cplx<T>);
 }
 template <typename T>
-size_t row_c2r_smem(const Geometry& g) {
-  return (size_t)2 * ((g.nx / 2 + 2) & ~1) * sizeof(cplx<T>) + 2 * padded_bytes(g.nx, sizeof(cplx<T>)) +
+size_t row_c2r_smem(const Geometry& g, int lb) {
+  return (size_t)(2 << lb) * ((g.nx / 2 + 2) & ~1) * sizeof(cplx<T>) + 2 * padded_bytes(g.nx << lb, sizeof(cplx<T>)) +
          (size_t)g.nx * sizeof(cplx<T>);
 }
 template <typename T>

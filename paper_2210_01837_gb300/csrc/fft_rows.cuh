@@ -7,10 +7,52 @@ namespace dps {
 
 template <typename T>
 bool fft_rows_allow() {
-  return allow_smem(row_r2c_kernel<T>) && allow_smem(row_c2r_kernel<T>) && allow_smem(row_r2c_reg_kernel<T, false>) &&
+  return allow_smem(row_r2c_kernel<T, false>) && allow_smem(row_c2r_kernel<T, false>) &&
+         allow_smem(row_r2c_kernel<T, true>) && allow_smem(row_c2r_kernel<T, true>) && allow_smem(row_r2c_reg_kernel<T, false>) &&
          allow_smem(row_r2c_reg_kernel<T, true>) && allow_smem(row_c2r_reg_kernel<T, false>) &&
          allow_smem(row_c2r_reg_kernel<T, true>);
 }
+
+namespace {
+
+// Share of the lanes that a block issues which carry butterflies, over all stages, with 2^lb row pairs.
+double lane_use(const FftPlan& fp, int lb) {
+  const int th = fft_threads(fp.n << lb);
+  double work = 0.0, issued = 0.0;
+  for (int s = 0; s < fp.nstages; ++s) {
+    const int bf = (fp.n << lb) / fp.radix[s], full = bf / th * th, rest = bf - full;
+    work += (double)bf * fp.radix[s];
+    issued += (double)(full + (rest + 31) / 32 * 32) * fp.radix[s];
+  }
+  return work / issued;
+}
+
+// log2 of the row pairs that a block of the shared-memory-staged passes transforms together (us of the
+// forward pass on 33 planes FP64 at 1, 2, 4 and 8 pairs, 97 planes float).
+//  - FP64: its instructions pay for idle lanes, so more pairs wherever they fill more of them, in at most 160
+//    threads; four rather than two below 1024 points, where the barriers are then shared by more work.
+//      64: 80 45 35 29   128: 182 106 80 84   210: 512 303 274 285   256: 559 344 309 311
+//      384: 823 852 756 825   675: 4012 3446 3689   1024: 5831 6509 6082
+//  - float: fours for short rows that leave a quarter of the lanes idle; longer rows, whose single-warp
+//    blocks run their barriers for free and whose epilogue reads without bank conflicts, stay single.
+//    (at 1 and 4 pairs) 64: 21 14   108: 33 31   160: 51 46   192: 68 55   200: 76 86   256: 93 101   384: 171 222
+// No more than leaves two units for every SM when three fields are transformed.
+template <typename T>
+int row_batch(const Geometry& g, const FftPlan& fp) {
+  int lb = 0;
+  if (sizeof(T) == 8) {
+    for (int l = 1; l <= 3 && (fp.n << l) <= 160 * kFftPer; ++l) {
+      const double ratio = lane_use(fp, l) / lane_use(fp, lb);
+      if (ratio > 1.04 || (lb == 1 && ratio > 0.999 && (fp.n << l) <= 1024)) lb = l;
+    }
+  } else if (fp.n <= 192 && lane_use(fp, 0) < 0.75) {
+    lb = 2;
+  }
+  while (lb > 0 && 3ll * g.nz * ((g.ny + (2 << lb) - 1) >> (lb + 1)) < 2 * 152) --lb;
+  return lb;
+}
+
+}  // namespace
 
 template <typename T>
 int fft_set_row_variant(Plan& p, int reg) {
@@ -25,12 +67,14 @@ int fft_set_row_variant(Plan& p, int reg) {
                                         : resident_grid(row_c2r_reg_kernel<T, false>, th, sm, p.device);
     return 1;
   }
-  const size_t r2c = row_r2c_smem<T>(p.g), c2r = row_c2r_smem<T>(p.g);
-  const int trow = fft_threads(p.g.nx);
+  const int lb = row_batch<T>(p.g, p.fx);
+  const size_t r2c = row_r2c_smem<T>(p.g, lb), c2r = row_c2r_smem<T>(p.g, lb);
+  const int trow = fft_threads(p.g.nx << lb);
   if (trow > kFftMaxThreads || r2c > 220 * 1024 || c2r > 220 * 1024) return 0;
   p.fft_reg[0] = 0;
-  p.fft_grid[0] = resident_grid(row_r2c_kernel<T>, trow, r2c, p.device);
-  p.fft_grid[1] = resident_grid(row_c2r_kernel<T>, trow, c2r, p.device);
+  p.row_lb = lb;
+  p.fft_grid[0] = resident_grid(lb ? row_r2c_kernel<T, true> : row_r2c_kernel<T, false>, trow, r2c, p.device);
+  p.fft_grid[1] = resident_grid(lb ? row_c2r_kernel<T, true> : row_c2r_kernel<T, false>, trow, c2r, p.device);
   return 1;
 }
 
@@ -78,13 +122,15 @@ void launch_fft_rows(const Plan& p, int dir, cudaStream_t s) {
       row_c2r_reg_kernel<T, false><<<p.fft_grid[1], th, sm, s>>>(g, p.fxr, twx, grid, p.zrange);
     return;
   }
-  const int th = fft_threads(g.nx);
-  if (dir < 0)
-    row_r2c_kernel<T><<<p.fft_grid[0], th, row_r2c_smem<T>(g), s>>>(g, p.fx, twx, reinterpret_cast<T*>(p.grid),
-                                                                      p.zrange);
-  else
-    row_c2r_kernel<T><<<p.fft_grid[1], th, row_c2r_smem<T>(g), s>>>(g, p.fx, twx, reinterpret_cast<T*>(p.grid),
-                                                                      p.zrange);
+  const int lb = p.row_lb, th = fft_threads(g.nx << lb);
+  T* grid = reinterpret_cast<T*>(p.grid);
+  if (dir < 0) {
+    const auto kernel = lb ? row_r2c_kernel<T, true> : row_r2c_kernel<T, false>;
+    kernel<<<p.fft_grid[0], th, row_r2c_smem<T>(g, lb), s>>>(g, p.fx, twx, grid, p.zrange, lb);
+  } else {
+    const auto kernel = lb ? row_c2r_kernel<T, true> : row_c2r_kernel<T, false>;
+    kernel<<<p.fft_grid[1], th, row_c2r_smem<T>(g, lb), s>>>(g, p.fx, twx, grid, p.zrange, lb);
+  }
 }
 
 }  // namespace dps
