@@ -1560,6 +1560,8 @@ void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s) {
   const LaneCfg fc = fwd_lane_cfg<T>(g);
   if (part != 1 && p.cheb_fold) {
     launch_cheb_fold(p, part == 2, kx0, w, s);
+  } else if (part != 1 && (p.cheb_columns & (part == 2 ? 2 : 1)) && (part == 2 || p.inject != 1)) {
+    launch_cheb_columns(p, part == 2, kx0, w, s);
   } else if (part == 0 && sizeof(T) == 4 && p.cheb_tc) {
     launch_cheb_fwd_tc(p, kx0, w, s);
   } else if (part == 0 && fc.threads > 0) {

@@ -336,8 +336,10 @@ dps_status allocate(Plan* p) {
   if (!cheb_tc_prepare(*p)) return DPS_ERR_CUDA;
   if (p->cheb_tc && !alloc((void**)&p->kt.bimg_f, cheb_tc_image_bytes(g, false))) return DPS_ERR_OOM;
   if (p->cheb_tc_bwd && !alloc((void**)&p->kt.bimg_b, cheb_tc_image_bytes(g, true))) return DPS_ERR_OOM;
+  p->cheb_columns = cheb_columns_applies(*p);
   if (const char* e = getenv("DPS_CHEB_TC")) {  // bit 0 forward, bit 1 backward
     const int v = atoi(e);
+    p->cheb_columns &= 2;
     p->cheb_tc = p->cheb_tc && (v & 1);
     p->cheb_tc_bwd = p->cheb_tc_bwd && (v & 2);
   }
@@ -666,14 +668,15 @@ dps_status dpstokes_plan_info(dps_plan_t plan, dps_plan_info* out) {
   // finishing kernel for the tile gather)
   // (+ the B-operand image kernel before each tensor-core transform)
   out->launches_per_apply = 9 + 5 * p->nchunks + ((p->interp_tile == 1 && p->ipart) ? 1 : 0) +
-                            p->nchunks * ((p->cheb_tc ? 1 : 0) + (p->cheb_tc_bwd ? 2 * p->cheb_tc_bwd_parts - 1 : 0));
+                            p->nchunks * ((p->cheb_tc && !(p->cheb_columns & 1) ? 1 : 0) +
+                                          (p->cheb_tc_bwd ? 2 * p->cheb_tc_bwd_parts - 1 : 0));
   out->nchunks = p->nchunks;
   out->fft_col_width = 1 << p->col_lcw;
   out->fft_register_rows = p->fft_reg[0];
   out->fft_register_cols = p->fft_reg[1];
   out->solve_blocks = p->bvp_blocks;
   out->interp_variant = p->interp_tile;
-  out->cheb_tensor_cores = (p->cheb_tc ? 1 : 0) | (p->cheb_tc_bwd ? 2 : 0);
+  out->cheb_tensor_cores = (p->cheb_tc && !(p->cheb_columns & 1) ? 1 : 0) | (p->cheb_tc_bwd ? 2 : 0);
   return DPS_OK;
 }
 
