@@ -91,8 +91,7 @@ struct Geometry {
   double uw0[2], uwH[2];
   int slip;
   int stage_cap;     // particle records the spreading kernel stages in shared memory at a time
-  int rec_threads;   // threads per block of the record kernel when it stages records in shared
-                     // memory (0: direct writes)
+  int rec_threads;   // threads per block of the thread-per-particle record kernel (0: records too large for it)
 };
 
 // Device tables owned by the plan

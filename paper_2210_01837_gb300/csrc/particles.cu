@@ -100,153 +100,285 @@ __device__ __forceinline__ int count_above(const double* zc, int nz, double v) {
   return lo;
 }
 
-// One thread per particle.  STAGED: the block's records are built in shared memory and then
-// copied to their contiguous place in global memory with 16-byte stores (a thread writing its own
-// record directly would make every warp store touch 32 different sectors).
-template <typename T, bool STAGED>
-__global__ void records_kernel(Geometry g, int64_t n, const double* __restrict__ pos,
-                               const double* __restrict__ F, const double* __restrict__ Tq,
-                               const double* __restrict__ zc, uint32_t* __restrict__ rec,
-                               int* __restrict__ bin_of, int* __restrict__ bin_count,
-                               int* __restrict__ zrange, int* __restrict__ status) {
-  extern __shared__ __align__(16) uint32_t srec_out[];
-  const int64_t j0 = (int64_t)blockIdx.x * blockDim.x;
-  const int64_t j = j0 + threadIdx.x;
-  if (!STAGED && j >= n) return;
-  if (j < n) {
-  uint32_t* r = STAGED ? srec_out + (size_t)threadIdx.x * g.rec_words : rec + (size_t)j * g.rec_words;
-  T* tv = reinterpret_cast<T*>(r + 8);
-  double x = pos[3 * j], y = pos[3 * j + 1], z = pos[3 * j + 2];
-  double f[3] = {F[3 * j], F[3 * j + 1], F[3 * j + 2]};
-  double tq[3] = {0.0, 0.0, 0.0};
-  if (g.with_torque) { tq[0] = Tq[3 * j]; tq[1] = Tq[3 * j + 1]; tq[2] = Tq[3 * j + 2]; }
-  bool finite = isfinite(x) && isfinite(y) && isfinite(z);
-  for (int i = 0; i < 3; ++i) finite = finite && isfinite(f[i]) && isfinite(tq[i]);
-  bool ok = finite;
-  if (!finite) atomicOr(status, kStatNonfinite);
+// A particle, checked (ok: finite and in the domain; else the status is set) and wrapped into the box
+struct RecParticle {
+  double x, y, z, f[3], tq[3];
+  bool ok;
+};
+__device__ __forceinline__ RecParticle rec_particle(const Geometry& g, int64_t j, const double* __restrict__ pos,
+                                                    const double* __restrict__ F, const double* __restrict__ Tq,
+                                                    int* __restrict__ status) {
+  RecParticle a;
+  const double x = pos[3 * j], y = pos[3 * j + 1];
+  a.z = pos[3 * j + 2];
+  for (int i = 0; i < 3; ++i) {
+    a.f[i] = F[3 * j + i];
+    a.tq[i] = g.with_torque ? Tq[3 * j + i] : 0.0;
+  }
+  bool ok = isfinite(x) && isfinite(y) && isfinite(a.z);
+  for (int i = 0; i < 3; ++i) ok = ok && isfinite(a.f[i]) && isfinite(a.tq[i]);
+  if (!ok) atomicOr(status, kStatNonfinite);
   double amax = g.kM.alpha;
   if (g.with_torque && g.kD.alpha > amax) amax = g.kD.alpha;
   if (ok) {
-    bool in_dom = (z >= g.zmin) && (z <= g.zmax);
-    if (g.mode == DPS_FREE && z - amax < g.zmin) in_dom = false;
-    if ((g.mode == DPS_FREE || g.mode == DPS_BOTTOM_WALL) && z + amax > g.zmax) in_dom = false;
+    bool in_dom = (a.z >= g.zmin) && (a.z <= g.zmax);
+    if (g.mode == DPS_FREE && a.z - amax < g.zmin) in_dom = false;
+    if ((g.mode == DPS_FREE || g.mode == DPS_BOTTOM_WALL) && a.z + amax > g.zmax) in_dom = false;
     if (!in_dom) { atomicOr(status, kStatDomain); ok = false; }
   }
   // wrap x, y into [0, L)
-  double xw = 0.0, yw = 0.0;
+  a.x = a.y = 0.0;
   if (ok) {
-    xw = x - g.Lx * floor(x / g.Lx);
-    if (xw >= g.Lx) xw -= g.Lx;
-    if (xw < 0.0) xw = 0.0;
-    yw = y - g.Ly * floor(y / g.Ly);
-    if (yw >= g.Ly) yw -= g.Ly;
-    if (yw < 0.0) yw = 0.0;
+    a.x = x - g.Lx * floor(x / g.Lx);
+    if (a.x >= g.Lx) a.x -= g.Lx;
+    if (a.x < 0.0) a.x = 0.0;
+    a.y = y - g.Ly * floor(y / g.Ly);
+    if (a.y >= g.Ly) a.y -= g.Ly;
+    if (a.y < 0.0) a.y = 0.0;
   }
-  const double tscale = g.torque_deriv ? 0.5 : 1.0;  // the derivative route stores tau / 2
+  a.ok = ok;
+  return a;
+}
+// force and torque at the head of the record's values (the derivative route stores tau / 2)
+template <typename T>
+__device__ __forceinline__ void rec_loads(const Geometry& g, const RecParticle& a, T* tv) {
+  const double tscale = g.torque_deriv ? 0.5 : 1.0;
   for (int i = 0; i < 3; ++i) {
-    tv[i] = ok ? (T)f[i] : (T)0;
-    tv[3 + i] = ok ? (T)(tscale * tq[i]) : (T)0;
+    tv[i] = a.ok ? (T)a.f[i] : (T)0;
+    tv[3 + i] = a.ok ? (T)(tscale * a.tq[i]) : (T)0;
   }
-  int cmin = g.nz, cmax = -1;
-  const int stride = 2 * g.pxc + g.lzc;
-  for (int K = 0; K < g.nkernels; ++K) {
-    const EsKernel& k = (K == 0) ? g.kM : g.kD;
-    int4 hd = make_int4(0, 0, 0, 0);
-    T* ph = tv + 6 + K * stride;
-    if (ok) {
-      const int ax = first_node(xw, g.h, g.inv_h, k.alpha);
-      const int ay = first_node(yw, g.h, g.inv_h, k.alpha);
-      const double tx0 = (double)ax * g.h - xw, ty0 = (double)ay * g.h - yw;  // offsets of the first nodes
-      {
-        double tx = tx0, ty = ty0;  // node offsets by running sums (one add each per slot)
-        for (int i = 0; i < g.pxc; ++i) {
-          ph[i] = (i < k.px) ? es_t<T>(tx, k) : (T)0;
-          ph[g.pxc + i] = (i < k.px) ? es_t<T>(ty, k) : (T)0;
-          tx += g.h;
-          ty += g.h;
-        }
-      }
-      hd.x = wrap_idx(ax, g.nx);
-      hd.y = wrap_idx(ay, g.ny);
-      // z support: nodes with z_c in [max(zmin, z - alpha), min(zmax, z + alpha)], widened by a
-      // hair so that the exact |t| <= alpha tests below decide membership
-      const double eps = 1e-12 * (g.H + fabs(z));
-      const int c0 = count_above(zc, g.nz, z + k.alpha + eps);
-      const int c1 = count_above(zc, g.nz, z - k.alpha - eps) - 1;
-      int cnt = c1 - c0 + 1;
-      if (cnt < 0) cnt = 0;
-      if (cnt > g.lzc) { cnt = g.lzc; atomicOr(status, kStatInternal); }
-      hd.z = c0;
-      hd.w = cnt;
-      const bool bottom_img = (g.mode == DPS_BOTTOM_WALL || g.mode == DPS_SLIT);
-      const bool top_img = (g.mode == DPS_SLIT);
-      for (int i = 0; i < g.lzc; ++i) {
-        T v = (T)0;
-        if (i < cnt) {
-          const double zz = zc[c0 + i];
-          T acc = es_t<T>(zz - z, k);
-          if (bottom_img) acc -= es_t<T>(zz - (2.0 * g.zmin - z), k);
-          if (top_img) acc -= es_t<T>(zz - (2.0 * g.zmax - z), k);
-          v = acc;
-        }
-        ph[2 * g.pxc + i] = v;
-      }
-      if (K == 1 && g.torque_deriv) {
-        // derivative slab: phi' in x and y, and d/dz of the imaged z factor (the exact derivative
-        // of the negatively imaged envelope)
-        T* pd = tv + 6 + 2 * stride;
-        double tx = tx0, ty = ty0;
-        for (int i = 0; i < g.pxc; ++i) {
-          pd[i] = (i < k.px) ? esd_t<T>(tx, k) : (T)0;
-          pd[g.pxc + i] = (i < k.px) ? esd_t<T>(ty, k) : (T)0;
-          tx += g.h;
-          ty += g.h;
-        }
-        for (int i = 0; i < g.lzc; ++i) {
-          T v = (T)0;
-          if (i < cnt) {
-            const double zz = zc[c0 + i];
-            T acc = esd_t<T>(zz - z, k);
-            if (bottom_img) acc -= esd_t<T>(zz - (2.0 * g.zmin - z), k);
-            if (top_img) acc -= esd_t<T>(zz - (2.0 * g.zmax - z), k);
-            v = acc;
-          }
-          pd[2 * g.pxc + i] = v;
-        }
-      }
-      if (cnt > 0) {
-        cmin = min(cmin, c0);
-        cmax = max(cmax, c0 + cnt - 1);
-      }
-    } else {
-      const int nv = (K == 1 && g.torque_deriv) ? 2 * stride : stride;  // slab K (and the derivatives)
-      for (int i = 0; i < nv; ++i) ph[i] = (T)0;
-    }
-    reinterpret_cast<int4*>(r)[K] = hd;
-  }
-  if (g.nkernels == 1) reinterpret_cast<int4*>(r)[1] = make_int4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void rec_bin(const Geometry& g, const RecParticle& a, int64_t j, int* __restrict__ bin_of,
+                                        int* __restrict__ bin_count) {
   int bx = 0, by = 0;
-  if (ok) {
-    bx = min((int)floor(xw * g.inv_h) / kTileX, g.nbx - 1);
-    by = min((int)floor(yw * g.inv_h) / kTileY, g.nby - 1);
+  if (a.ok) {
+    bx = min((int)floor(a.x * g.inv_h) / kTileX, g.nbx - 1);
+    by = min((int)floor(a.y * g.inv_h) / kTileY, g.nby - 1);
   }
   const int b = by * g.nbx + bx;
   bin_of[j] = b;
   atomicAdd(&bin_count[b], 1);
-  if (cmax >= 0) {
+}
+// z support: nodes with z_c in [max(zmin, z - alpha), min(zmax, z + alpha)], widened by a hair so that the exact
+// |t| <= alpha tests decide membership; returns their number
+__device__ __forceinline__ int rec_zsupport(const Geometry& g, const EsKernel& k, const double* zc, double z, int& c0,
+                                            int* __restrict__ status) {
+  const double eps = 1e-12 * (g.H + fabs(z));
+  c0 = count_above(zc, g.nz, z + k.alpha + eps);
+  const int c1 = count_above(zc, g.nz, z - k.alpha - eps) - 1;
+  int cnt = c1 - c0 + 1;
+  if (cnt < 0) cnt = 0;
+  if (cnt > g.lzc) { cnt = g.lzc; atomicOr(status, kStatInternal); }
+  return cnt;
+}
+
+// A block builds the records of P particles (P a power of two, at most kRecMax): a thread per particle and
+// record head checks the particle, finds its support and forms the node offsets by running sums (one add each
+// per slot), then all threads evaluate the envelope, a thread per value, and write the records with contiguous
+// stores.  Few particles are bound by the chain of a value (some hundred instructions in double), which a
+// thread per particle runs once per slot; many in double or with derivatives by the FP64 pipe, which then has no
+// idle lanes at the images and the shorter supports.  Against a thread per particle: 100 spheres in double 75 ->
+// 14 us, 1001 with torques 92 -> 20, 317 mixed 25 -> 12, 16384 in double 205 -> 172, 16384 mixed 43 -> 27, 262144
+// with derivatives 315 -> 209.
+constexpr int kRecThreads = 128, kRecMax = 32, kRecNodes = 512;  // kRecNodes: nodes copied to shared memory
+
+// doubles of a particle's running offsets in shared memory (odd: consecutive particles in different banks)
+__host__ __device__ inline int rec_offsets(const Geometry& g) { return 2 * g.pxc + 1; }
+__host__ __device__ inline size_t rec_smem(const Geometry& g, int P) {
+  return ((size_t)(g.nz <= kRecNodes ? g.nz : 0) + (size_t)P * (g.nkernels * rec_offsets(g) + 3)) * sizeof(double) +
+         (size_t)2 * P * g.nkernels * sizeof(int);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRecThreads) records_kernel(Geometry g, int64_t n, const double* __restrict__ pos,
+                                                              const double* __restrict__ F,
+                                                              const double* __restrict__ Tq,
+                                                              const double* __restrict__ zc_g,
+                                                              uint32_t* __restrict__ rec, int* __restrict__ bin_of,
+                                                              int* __restrict__ bin_count, int* __restrict__ zrange,
+                                                              int* __restrict__ status, int P) {
+  extern __shared__ __align__(16) double rec_sm[];
+  const int nk = g.nkernels, no = rec_offsets(g), tid = threadIdx.x;
+  double* offs = rec_sm;                     // [nk][P][no] x offsets, then y offsets
+  double* zz3 = offs + (size_t)nk * P * no;  // [P][3] z and its images at the walls
+  double* zn = zz3 + 3 * P;                  // [nz] the nodes
+  int* c0s = reinterpret_cast<int*>(zn + (g.nz <= kRecNodes ? g.nz : 0));  // [nk][P] first node
+  int* cnts = c0s + nk * P;                                                // [nk][P] nodes; -1: not in the domain
+  const int64_t j0 = (int64_t)blockIdx.x * P;
+  if (g.nz <= kRecNodes)
+    for (int i = tid; i < g.nz; i += kRecThreads) zn[i] = zc_g[i];
+  const double* zc = g.nz <= kRecNodes ? zn : zc_g;
+  __syncthreads();
+  const int heads = P < kRecMax ? nk : 1;  // threads per particle: one where the FP64 pipe, not latency, is the bound
+  int cmin = g.nz, cmax = -1;
+  if (tid < P * heads && j0 + (tid & (P - 1)) < n) {
+    const int p = tid & (P - 1), K0 = tid >= P;
+    const int64_t j = j0 + p;
+    uint32_t* r = rec + (size_t)j * g.rec_words;
+    const RecParticle a = rec_particle(g, j, pos, F, Tq, status);
+    for (int K = K0; K < nk; K += heads) {
+      int4 hd = make_int4(0, 0, 0, 0);
+      int cnt = -1;
+      if (a.ok) {
+        const EsKernel& k = (K == 0) ? g.kM : g.kD;
+        const int ax = first_node(a.x, g.h, g.inv_h, k.alpha);
+        const int ay = first_node(a.y, g.h, g.inv_h, k.alpha);
+        double tx = (double)ax * g.h - a.x, ty = (double)ay * g.h - a.y;  // offsets of the first nodes
+        double* o = offs + (size_t)(K * P + p) * no;
+        for (int i = 0; i < g.pxc; ++i) {
+          o[i] = tx;
+          o[g.pxc + i] = ty;
+          tx += g.h;
+          ty += g.h;
+        }
+        int c0;
+        cnt = rec_zsupport(g, k, zc, a.z, c0, status);
+        hd = make_int4(wrap_idx(ax, g.nx), wrap_idx(ay, g.ny), c0, cnt);
+        if (cnt > 0) {
+          cmin = min(cmin, c0);
+          cmax = max(cmax, c0 + cnt - 1);
+        }
+        c0s[K * P + p] = c0;
+      }
+      cnts[K * P + p] = cnt;
+      reinterpret_cast<int4*>(r)[K] = hd;
+    }
+    if (K0 == 0) {
+      if (nk == 1) reinterpret_cast<int4*>(r)[1] = make_int4(0, 0, 0, 0);
+      rec_loads(g, a, reinterpret_cast<T*>(r + 8));
+      zz3[3 * p] = a.z;
+      zz3[3 * p + 1] = 2.0 * g.zmin - a.z;
+      zz3[3 * p + 2] = 2.0 * g.zmax - a.z;
+      rec_bin(g, a, j, bin_of, bin_count);
+    }
+  }
+  cmin = __reduce_min_sync(0xffffffffu, cmin);
+  cmax = __reduce_max_sync(0xffffffffu, cmax);
+  if ((tid & 31) == 0 && cmax >= 0) {
     atomicMin(&zrange[0], cmin);
     atomicMax(&zrange[1], cmax);
   }
-  }  // j < n
-  if (STAGED) {
-    __syncthreads();
-    const int64_t left = n - j0;
-    const int cnt = left < (int64_t)blockDim.x ? (int)left : (int)blockDim.x;
-    const int q = cnt * (g.rec_words / 4);  // 16-byte pieces (rec_words is a multiple of 4)
-    const uint4* src = reinterpret_cast<const uint4*>(srec_out);
-    uint4* dst = reinterpret_cast<uint4*>(rec + (size_t)j0 * g.rec_words);
-    for (int t = threadIdx.x; t < q; t += blockDim.x) dst[t] = src[t];
+  __syncthreads();
+  const int stride = 2 * g.pxc + g.lzc, live = (int)min((int64_t)P, n - j0);
+  const bool bottom_img = (g.mode == DPS_BOTTOM_WALL || g.mode == DPS_SLIT), top_img = (g.mode == DPS_SLIT);
+  for (int K = 0; K < nk; ++K) {
+    const EsKernel& k = (K == 0) ? g.kM : g.kD;
+    const bool deriv = K == 1 && g.torque_deriv;
+    // slot e of particle p: this thread's slots are kRecThreads apart
+    auto each = [&](int per, auto&& slot) {
+      const int dp = kRecThreads / per, de = kRecThreads - dp * per;
+      int p = tid / per, e = tid - p * per;
+      while (p < live) {
+        T* ph = reinterpret_cast<T*>(rec + (size_t)(j0 + p) * g.rec_words + 8) + 6 + K * stride;
+        slot(p, e, ph);
+        p += dp;
+        e += de;
+        if (e >= per) {
+          e -= per;
+          ++p;
+        }
+      }
+    };
+    each(2 * g.pxc, [&](int p, int e, T* ph) {
+      const bool in = cnts[K * P + p] >= 0 && (e < g.pxc ? e : e - g.pxc) < k.px;
+      const double t = in ? offs[(size_t)(K * P + p) * no + e] : 0.0;
+      ph[e] = in ? es_t<T>(t, k) : (T)0;
+      if (deriv) ph[stride + e] = in ? esd_t<T>(t, k) : (T)0;  // phi' in x and y
+    });
+    each(g.lzc, [&](int p, int i, T* ph) {
+      T v = (T)0, d = (T)0;
+      if (i < cnts[K * P + p]) {
+        const double zz = zc[c0s[K * P + p] + i], t = zz - zz3[3 * p];
+        v = es_t<T>(t, k);
+        if (deriv) d = esd_t<T>(t, k);
+        if (bottom_img) {
+          const double tb = zz - zz3[3 * p + 1];
+          v -= es_t<T>(tb, k);
+          if (deriv) d -= esd_t<T>(tb, k);
+        }
+        if (top_img) {
+          const double tt = zz - zz3[3 * p + 2];
+          v -= es_t<T>(tt, k);
+          if (deriv) d -= esd_t<T>(tt, k);
+        }
+      }
+      ph[2 * g.pxc + i] = v;
+      // d/dz of the imaged z factor (the exact derivative of the negatively imaged envelope)
+      if (deriv) ph[stride + 2 * g.pxc + i] = d;
+    });
   }
+}
+
+// Many particles in mixed precision without derivatives: one thread per particle, whose values cost little more
+// than their bookkeeping above (a million with torques: 627 us here, 692 there).  The block's records are built
+// in shared memory and then copied to their contiguous place in global memory with 16-byte stores (a thread
+// writing its own record directly would make every warp store touch 32 different sectors).
+__global__ void records_thread_kernel(Geometry g, int64_t n, const double* __restrict__ pos,
+                                      const double* __restrict__ F, const double* __restrict__ Tq,
+                                      const double* __restrict__ zc, uint32_t* __restrict__ rec,
+                                      int* __restrict__ bin_of, int* __restrict__ bin_count, int* __restrict__ zrange,
+                                      int* __restrict__ status) {
+  extern __shared__ __align__(16) uint32_t srec_out[];
+  const int64_t j0 = (int64_t)blockIdx.x * blockDim.x;
+  const int64_t j = j0 + threadIdx.x;
+  if (j < n) {
+    uint32_t* r = srec_out + (size_t)threadIdx.x * g.rec_words;
+    float* tv = reinterpret_cast<float*>(r + 8);
+    const RecParticle a = rec_particle(g, j, pos, F, Tq, status);
+    rec_loads(g, a, tv);
+    int cmin = g.nz, cmax = -1;
+    const int stride = 2 * g.pxc + g.lzc;
+    const bool bottom_img = (g.mode == DPS_BOTTOM_WALL || g.mode == DPS_SLIT), top_img = (g.mode == DPS_SLIT);
+    for (int K = 0; K < g.nkernels; ++K) {
+      const EsKernel& k = (K == 0) ? g.kM : g.kD;
+      int4 hd = make_int4(0, 0, 0, 0);
+      float* ph = tv + 6 + K * stride;
+      if (a.ok) {
+        const int ax = first_node(a.x, g.h, g.inv_h, k.alpha);
+        const int ay = first_node(a.y, g.h, g.inv_h, k.alpha);
+        double tx = (double)ax * g.h - a.x, ty = (double)ay * g.h - a.y;  // node offsets by running sums
+        for (int i = 0; i < g.pxc; ++i) {
+          ph[i] = (i < k.px) ? es_eval_f(tx, k) : 0.f;
+          ph[g.pxc + i] = (i < k.px) ? es_eval_f(ty, k) : 0.f;
+          tx += g.h;
+          ty += g.h;
+        }
+        int c0;
+        const int cnt = rec_zsupport(g, k, zc, a.z, c0, status);
+        hd = make_int4(wrap_idx(ax, g.nx), wrap_idx(ay, g.ny), c0, cnt);
+        for (int i = 0; i < g.lzc; ++i) {
+          float v = 0.f;
+          if (i < cnt) {
+            const double zz = zc[c0 + i];
+            v = es_eval_f(zz - a.z, k);
+            if (bottom_img) v -= es_eval_f(zz - (2.0 * g.zmin - a.z), k);
+            if (top_img) v -= es_eval_f(zz - (2.0 * g.zmax - a.z), k);
+          }
+          ph[2 * g.pxc + i] = v;
+        }
+        if (cnt > 0) {
+          cmin = min(cmin, c0);
+          cmax = max(cmax, c0 + cnt - 1);
+        }
+      } else {
+        for (int i = 0; i < stride; ++i) ph[i] = 0.f;
+      }
+      reinterpret_cast<int4*>(r)[K] = hd;
+    }
+    if (g.nkernels == 1) reinterpret_cast<int4*>(r)[1] = make_int4(0, 0, 0, 0);
+    rec_bin(g, a, j, bin_of, bin_count);
+    if (cmax >= 0) {
+      atomicMin(&zrange[0], cmin);
+      atomicMax(&zrange[1], cmax);
+    }
+  }
+  __syncthreads();
+  const int64_t left = n - j0;
+  const int cnt = left < (int64_t)blockDim.x ? (int)left : (int)blockDim.x;
+  const int q = cnt * (g.rec_words / 4);  // 16-byte pieces (rec_words is a multiple of 4)
+  const uint4* src = reinterpret_cast<const uint4*>(srec_out);
+  uint4* dst = reinterpret_cast<uint4*>(rec + (size_t)j0 * g.rec_words);
+  for (int t = threadIdx.x; t < q; t += blockDim.x) dst[t] = src[t];
 }
 
 // exclusive scan of bin counts (one block of 32 warps; bins in contiguous chunks per thread, four at a time):
@@ -1848,18 +1980,27 @@ dps_status particle_geometry(Geometry& g, const dps_kernel_params* kp, int tsize
   return DPS_OK;
 }
 
+// particles from which the thread-per-particle kernel is the faster one (mixed, no derivatives, us against
+// records_kernel: 16384 43 / 27, 65536 55 / 60, 1048576 627 / 692; one head: 32768 18 / 18, 663552 155 / 180)
+constexpr int64_t kRecThreadMin = 49152;
+
 template <typename T>
 void launch_records(const Plan& p, int64_t n, const double* pos, const double* F, const double* Tq,
                     cudaStream_t s) {
   if (n <= 0) return;
-  const int threads = p.g.rec_threads > 0 ? p.g.rec_threads : 128;
-  const unsigned blocks = (unsigned)((n + threads - 1) / threads);
-  if (p.g.rec_threads > 0)
-    records_kernel<T, true><<<blocks, threads, (size_t)threads * p.g.rec_words * sizeof(uint32_t), s>>>(
+  if (sizeof(T) == 4 && !p.g.torque_deriv && p.g.rec_threads > 0 && n >= kRecThreadMin) {
+    const int threads = p.g.rec_threads;
+    records_thread_kernel<<<(unsigned)((n + threads - 1) / threads), threads,
+                            (size_t)threads * p.g.rec_words * sizeof(uint32_t), s>>>(
         p.g, n, pos, F, Tq, p.tab.zc, p.records, p.bin_of, p.bin_count, p.zrange, p.status);
-  else
-    records_kernel<T, false><<<blocks, threads, 0, s>>>(p.g, n, pos, F, Tq, p.tab.zc, p.records, p.bin_of,
-                                                        p.bin_count, p.zrange, p.status);
+    return;
+  }
+  // as many particles per block as leave two blocks for every SM, and fit in the default shared memory (one
+  // always does: supports are at most 80 nodes wide)
+  int P = kRecMax;
+  while (P > 1 && (n < (int64_t)P * 2 * 152 || rec_smem(p.g, P) > 48 * 1024)) P /= 2;
+  records_kernel<T><<<(unsigned)((n + P - 1) / P), kRecThreads, rec_smem(p.g, P), s>>>(
+      p.g, n, pos, F, Tq, p.tab.zc, p.records, p.bin_of, p.bin_count, p.zrange, p.status, P);
 }
 
 void launch_bins(const Plan& p, int64_t n, cudaStream_t s) {
@@ -1909,9 +2050,9 @@ int spread_prepare(Plan& p) {
   const long rb = (long)p.g.rec_words * (long)sizeof(uint32_t);
   const long cap = ((long)optin - (long)std::max(fa.sharedSizeBytes, fi.sharedSizeBytes)) / rb;
   p.g.stage_cap = (int)std::min<long>(kStage, cap);
-  // records built in shared memory by blocks of 128, 64 or 32 threads when that many fit in
-  // 96 KB (two blocks per SM), else written directly
-  if (!allow_smem(records_kernel<T, true>)) return 0;
+  // records built in shared memory by blocks of 128, 64 or 32 threads when that many fit in 96 KB (two blocks
+  // per SM)
+  if (!allow_smem(records_thread_kernel)) return 0;
   p.g.rec_threads = 0;
   for (int t : {128, 64, 32})
     if ((long)t * rb <= 96 * 1024) { p.g.rec_threads = t; break; }
