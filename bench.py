@@ -690,10 +690,10 @@ def main():
                            "frac_fp64_nominal": round(solve_tflops / FP64_NOMINAL_TFLOPS, 3)}
     dom = max((k for k in stages if k in work or k == "solve"), key=stages.get)
     if dom == "solve":
-        roofline = {"bound": "alu", "kernel": "solve_tab_kernel (FP64 banded solves)", "achieved": round(solve_tflops, 4),
+        roofline = {"bound": "alu", "kernel": "solve_tile_kernel (banded solves)", "achieved": round(solve_tflops, 4),
                     "peak": round(FP64_NOMINAL_TFLOPS, 3), "unit": "TFLOP/s",
                     "frac": round(solve_tflops / FP64_NOMINAL_TFLOPS, 4),
-                    "traffic": measured_traffic("solve_tab_kernel<float, 0>") if div == 1 and not args.nz else None,
+                    "traffic": measured_traffic("solve_tile_kernel<float, 0>") if div == 1 and not args.nz else None,
                     "traffic_source": "profiles/traffic.json (ncu dram bytes, scaled by wavenumbers)",
                     "peak_kind": "FP64 nominal from unit counts x max clock"}
     else:

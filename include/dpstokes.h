@@ -48,8 +48,9 @@ typedef enum {
 typedef enum {
   DPS_FP64 = 0,   /* every stage in double precision                                           */
   DPS_MIXED = 1   /* spreading, FFTs, Chebyshev transforms, interpolation in float (float
-                     accumulation); the banded BVP solves and the wall-correction boundary rows
-                     in double                                                                   */
+                     accumulation); the wall-correction boundary rows and the factorisation of
+                     the banded BVP solves in double, their sweeps in double or in 64-bit fixed
+                     point                                                                       */
 } dps_precision;
 
 /* how torques enter (the two routes of Sec. III.D, the paragraph after the algorithm) */
@@ -225,7 +226,7 @@ dps_status dpstokes_plan_autotune(dps_plan_t plan, int64_t n, const double* posi
 dps_status dpstokes_plan_set_fft(dps_plan_t plan, int32_t row_register, int32_t col_register, int32_t col_width);
 
 /* Sets the wavenumber-space pipeline shape by hand (no counterpart in the paper): `solve_blocks`
- * persistent blocks of the FP64 solve (1 .. the number the plan's workspace was sized for, which
+ * persistent blocks of the FP64 solve (1 .. the number the plan was made for, which
  * dpstokes_plan_info reports as solve_blocks right after creation) and `nchunks` column chunks
  * (1, 2, 4 or 8, at least 64 x-wavenumbers each) whose FP64 solves run on a plan-owned stream
  * beside the float transforms of the neighbouring chunks.  Results do not depend on the shape

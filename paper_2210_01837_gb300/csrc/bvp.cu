@@ -1,4 +1,6 @@
-// Per-wavenumber stage of the doubly-periodic Stokes solve (steps 2-7 of Sec. III.D, z part).
+// Per-wavenumber stage of the doubly-periodic Stokes solve (steps 2-7 of Sec. III.D, z part): the forms that
+// take every plan, and the dispatch to the specialised ones (the tiled solve in solve.cu; transforms on the
+// tensor cores in cheb_tc.cu, by folding in cheb_fold.cu, in registers in cheb_columns.cu).
 //
 // Three kernels, each shaped for the pipe it needs, with one thread per (kx, ky) of the half
 // spectrum and k-contiguous (coalesced) layouts throughout:
