@@ -338,6 +338,7 @@ __device__ __noinline__ void zero_mode_warp(const Geometry& g, const double* __r
                                             cplx<T>* __restrict__ kaux, cplx<double>* __restrict__ sc, int64_t K) {
   const int N = g.nz, lane = threadIdx.x & 31;
   const double *bl = band, *bd = band + N, *bu = band + 2 * N, *bP = band + 3 * N, *bQ = band + 4 * N;
+  __syncwarp();  // sc is the warp's slab: its sweeps have read their columns before other lanes write over them
   auto sum = [](cplx<double> v) {
     for (int o = 16; o; o >>= 1) {
       v.x += __shfl_xor_sync(0xffffffffu, v.x, o);

@@ -6,6 +6,7 @@ the oracle at the parity bars (1e-9 in double, 1e-5 in mixed precision)."""
 import pytest
 
 from oracle.stokes import mobility
+from paper_2210_01837_gb300 import binding
 from paper_2210_01837_gb300.workloads import random_particles
 from gpu_helpers import gpu_mobility, oracle_params, rel_l2, small_params
 
@@ -27,3 +28,27 @@ def test_tiled_solve_at_the_edges_matches_oracle(nx, ny, nz, zmax, mode, precisi
     U, W = gpu_mobility(params, pos, F, T, precision)
     assert rel_l2(U, U_ref) <= TOL[precision]
     assert rel_l2(W, W_ref) <= TOL[precision]
+
+
+# slip lengths and wall velocities: the wall rows of k = 0 as well as those of every other wavenumber
+WALLS = dict(slip_bottom=0.4, slip_top=0.7, uw_bottom=(0.3, -0.2), uw_top=(-0.5, 0.6))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("nx,ny,nz,zmax", [(27, 25, 34, 6.0), (40, 36, 33, 6.0)])
+def test_one_block_runs_all_tiles_and_the_zero_mode(nx, ny, nz, zmax, precision):
+    """22 and 48 tiles in one block: the rings of constants (16 tiles) and of wall values (9) wrap, and the
+    zero mode, on a warp between two of its tiles, takes that warp's shared memory for a while.  The
+    wavenumbers are independent, so the result is that of the default grid bit for bit."""
+    params = small_params("slit", nx=nx, ny=ny, nz=nz, zmax=zmax, torque=True)
+    params.update(WALLS)
+    pos, F, T = random_particles(params, 9, seed=nx)
+    U_ref, W_ref = mobility(oracle_params(params), pos, F, T)
+    plan = binding.Plan.from_params(params, with_torque=True, precision=precision, max_n=len(pos))
+    U0, W0 = gpu_mobility(params, pos, F, T, precision, plan=plan)
+    plan.set_pipeline(1, 1)
+    U1, W1 = gpu_mobility(params, pos, F, T, precision, plan=plan)
+    plan.close()
+    assert rel_l2(U0, U_ref) <= TOL[precision]
+    assert rel_l2(W0, W_ref) <= TOL[precision]
+    assert (U1 == U0).all() and (W1 == W0).all()
