@@ -48,9 +48,8 @@ typedef enum {
 typedef enum {
   DPS_FP64 = 0,   /* every stage in double precision                                           */
   DPS_MIXED = 1   /* spreading, FFTs, Chebyshev transforms, interpolation in float (float
-                     accumulation); the wall-correction boundary rows and the factorisation of
-                     the banded BVP solves in double, their sweeps in double or in 64-bit fixed
-                     point                                                                       */
+                     accumulation); the banded BVP solves and the wall-correction boundary rows
+                     in double                                                                   */
 } dps_precision;
 
 /* how torques enter (the two routes of Sec. III.D, the paragraph after the algorithm) */

@@ -13,9 +13,11 @@
 // 1.3 GB at 768 x 768 x 65 (spectra and table).
 //
 // Measured (solve alone, GB300, thread per wavenumber -> this): 120 x 120 x 33 mixed 155 -> 47 us,
-// 128 x 128 x 65 double 430 -> 159 us, 768 x 768 x 65 mixed 1.73 -> 1.41
-// ms, 3072 x 3072 x 65 mixed 23.3 -> 22.2 ms.  It is bound by latency: 16 warps an SM (the slabs' shared
-// memory), issue slots 47 % and the FP64 pipe 45 % busy.
+// 128 x 128 x 65 double 434 -> 172 us, 768 x 768 x 65 mixed 1.72 -> 1.40 ms, 3072 x 3072 x 65 mixed
+// 23.2 -> 22.3 ms.  It is bound by latency: 16 warps an SM (the slabs' shared memory).  The sweeps run in
+// double in float plans too, as the boundary sums do: 64-bit fixed-point sweeps on the integer pipe took the
+// same time (1.40 and 22.3 ms), lost bits in the small entries of a column and turned an overflow into
+// finite numbers.
 #include "bvp_device.cuh"
 #include "dps_internal.cuh"
 
@@ -76,42 +78,6 @@ __device__ __forceinline__ SolveSmem<T> solve_smem(unsigned char* base, int N, b
   return m;
 }
 
-// ---------------------------------------------------------------------------------------------
-// 64-bit fixed point, for the sweeps of float plans.  Their recurrences are the only serial part of a
-// system and need nothing of a floating exponent once the largest right-hand side is known, and the
-// integer pipe runs them at twice the rate of the FP64 pipe and beside it (measured per clock and SM:
-// DFMA 1.9, this product 3.9), so the FP64 pipe keeps the wall and boundary sums alone.  A value is
-// an int64 times 2^(E - 55), 2^E above the largest magnitude: the rounding error of a step is 2^-53 of that
-// magnitude or less, the unit roundoff of a double at it.  The factors are below 4 in magnitude and
-// stored as int64 times 2^-60.
-// ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ double ldexp_small(double v, int k) { return v * __hiloint2double((k + 1023) << 20, 0); }
-
-// v f / 2^60, dropping the product of the (signed) low halves: at most 4 units of 2^-62 of the range
-// the factor's halves are stored as signed numbers, f = fh 2^32 + fl
-__device__ __forceinline__ long long fx_mul(long long v, int2 f) {
-  const int vl = (int)v;
-  const int vh = (int)((v + 0x80000000ll) >> 32);
-  const long long m = (long long)vh * f.x + (long long)vl * f.y;
-  return (((long long)vh * f.y) << 4) + (m >> 28);
-}
-
-// int64 -> float by its halves: a 64-bit conversion would run on the FP64 pipe
-__device__ __forceinline__ float fx_float(long long v) {
-  return fmaf((float)(int)(v >> 32), 4294967296.0f, (float)(unsigned)v);
-}
-
-// float -> fixed point with biased exponent e of 2^E (r below 2^E in magnitude): r 2^(55 - E)
-__device__ __forceinline__ long long fx_from(float r, int e) {
-  const int b = __float_as_int(r);
-  const int eb = (b >> 23) & 0xff;
-  int mant = (b & 0x7fffff) | 0x800000;
-  if (eb == 0) mant = 0;  // zero (float subnormals flush to zero, as everywhere in the solve)
-  if (b < 0) mant = -mant;
-  const int d = e - eb;  // >= 1
-  return ((long long)mant << 32) >> (d < 63 ? d : 63);
-}
-
 // Rows in two batches of B in registers: while the rows of one are used, the loads of the other are in
 // flight (a batch's loads are waited for together, so rows ahead of it never hold a wait back).  Rows run
 // from `from` to `to` (at least one) in steps of D (1 or -1); load(r, more) reads the next row and, with
@@ -148,8 +114,8 @@ template <typename T>
 struct SolveTable {
   double2* gw;     // [N][KP]
   double* edge;    // [2][7][KP]
-  int2* V;         // [N][KP] fixed point (low, high half; float plans) or the bits of a double
-  int2* t;         // [N][KP]
+  double* V;       // [N][KP]
+  double* t;       // [N][KP]
   double* wd;      // [N][KP], slip only
   T* rho;          // [N][KP]
   int64_t KP;
@@ -168,9 +134,9 @@ __host__ inline SolveTable<T> solve_table(const Plan& p) {
   t.KP = p.kt.KP;
   t.gw = reinterpret_cast<double2*>(p.kt.fac);
   t.edge = reinterpret_cast<double*>(t.gw + n);
-  t.V = reinterpret_cast<int2*>(t.edge + 14 * (size_t)t.KP);
+  t.V = t.edge + 14 * (size_t)t.KP;
   t.t = t.V + n;
-  t.wd = p.g.slip ? reinterpret_cast<double*>(t.t + n) : nullptr;
+  t.wd = p.g.slip ? t.t + n : nullptr;
   t.rho = p.g.slip ? reinterpret_cast<T*>(t.wd + n) : reinterpret_cast<T*>(t.t + n);
   return t;
 }
@@ -180,7 +146,7 @@ template <typename T>
 struct Rows {
   const double2* gw;      // gamma, omega
   const double* wd;       // omega of the derivative (slip)
-  const int2 *V, *t;      // -V_n and -t_n
+  const double *V, *t;    // -V_n and -t_n
   const T* rho;
   int64_t KP;
 };
@@ -192,21 +158,21 @@ __device__ __forceinline__ Rows<T> SolveTable<T>::rows(int par, int kp) const {
 }
 
 // A real system takes three passes.  Pass 1 forms the scaled right-hand sides r'_i = r_i rho_i in the transform precision
-// (rhs(i, x) from the values that load(i, x) fetched), keeps them in the slab and adds up the boundary
+// (rhs(i, x) from the values that load(i, x) fetched), keeps them in the slab, widened, and adds up the boundary
 // row and the wall value as functionals of them, in double: g -= sum gamma_i r'_i, q = sum omega_i r'_i
 // (adjoints of the two sweeps, formed when the plan is made).  These sums have no serial part, so a warp
 // can fill its FP64 pipe.  Pass 2 is the elimination s_i = r'_i - V_i s_{i+1}, i = il .. 1, pass 3 the
 // substitution (sweeps).
 template <typename T, bool SLIP, typename In, typename Load, typename Rhs>
-__device__ __forceinline__ void functionals(int il, const Rows<T>& tb, unsigned char* slab, int lane, double& g, double& q,
-                                            double& qd, T& mx, Load&& load, Rhs&& rhs) {
+__device__ __forceinline__ void functionals(int il, const Rows<T>& tb, double* slab, int lane, double& g, double& q,
+                                            double& qd, Load&& load, Rhs&& rhs) {
   struct Row {
     double2 gw;
     double wd;
     T rho;
     In in;
   };
-  T* rr = reinterpret_cast<T*>(slab) + lane;
+  double* rr = slab + lane;
   const size_t st = 2 * (size_t)tb.KP;
   const double2* pg = tb.gw + il * st;
   const double* pw = SLIP ? tb.wd + il * st : nullptr;
@@ -222,105 +188,63 @@ __device__ __forceinline__ void functionals(int il, const Rows<T>& tb, unsigned 
     }
     load(x.in, more);
   };
-  mx = (T)0;
   Row x[3];
   rows_fetch<3, -1, Row>(x, il, 1, fetch);
   rows_ahead<3, -1, Row>(x, il, 1, fetch, [&](int i, const Row& v) {
-    const T r = rhs(i, v.in) * v.rho;
-    rr[i * 32] = r;
-    mx = fmax(mx, fabs(r));
-    const double d = widen<T>(r);
+    const double d = widen<T>(rhs(i, v.in) * v.rho);
+    rr[i * 32] = d;
     g = fma(-v.gw.x, d, g);
     q = fma(v.gw.y, d, q);
     if (SLIP) qd = fma(v.wd, d, qd);
   });
 }
 
-__device__ __forceinline__ double as_double(int2 v) { return __hiloint2double(v.y, v.x); }
-
 // Passes 2 and 3 of a system: the elimination in place and s_1 from it, the 2 x 2 boundary system for c_0 and
 // a, and the substitution c_i = s_i - t_i c_{i-1} with y = B B c (+ a in row 0) handed to put(i, y) in the
 // transform precision.  Returns the wall value's and (qd) the wall derivative's part of this parity.
 template <typename T, bool SLIP, typename Put>
 __device__ __forceinline__ double sweeps(int il, int par, const Rows<T>& tb, const double* __restrict__ edge,
-                                         unsigned char* slab, int lane, const SolveSmem<T>& m, T mx, T r0, double g,
-                                         double q, double& qd, Put&& put) {
+                                         double* slab, int lane, const SolveSmem<T>& m, T r0, double g, double q,
+                                         double& qd, Put&& put) {
   const size_t st = 2 * (size_t)tb.KP;
   const int64_t KP = tb.KP;
-  const int2* pv = tb.V + il * st;
-  const int2* pt = tb.t + st;
-  auto fv = [&](int2& x, bool more) {
+  const double* pv = tb.V + il * st;
+  const double* pt = tb.t + st;
+  auto fv = [&](double& x, bool more) {
     x = *pv;
     if (more) pv -= st;
   };
-  auto ft = [&](int2& x, bool more) {
+  auto ft = [&](double& x, bool more) {
     x = *pt;
     if (more) pt += st;
   };
-  int2 v[4], t[4];
-  rows_fetch<4, -1, int2>(v, il, 1, fv);
+  double v[4], t[4];
+  rows_fetch<4, -1, double>(v, il, 1, fv);
   const double U = edge[0], cb = edge[KP], ck = edge[2 * KP], cd = edge[3 * KP], cc = edge[4 * KP], w0 = edge[5 * KP];
   const double w0d = SLIP ? edge[6 * KP] : 0.0;
-  rows_fetch<4, 1, int2>(t, 1, il, ft);
-  T c2 = (T)0, c1, sc = (T)1, ta;
+  rows_fetch<4, 1, double>(t, 1, il, ft);
+  double* sw = slab + lane;
+  double s = 0.0;
+  rows_ahead<4, -1, double>(v, il, 1, fv, [&](int i, double f) {
+    s = fma(f, s, sw[i * 32]);
+    sw[i * 32] = s;
+  });
+  const double rh = fma(-s, U, widen<T>(r0));
+  const double c0 = fma(g, ck, rh * cb), a = fma(g, cd, -(rh * cc));
+  const T ta = narrow<T>(a);
+  T c2 = (T)0, c1 = narrow<T>(c0);
   auto row = [&](int i, T cn) {  // row i of y, whose neighbours c_{i-1} and c_{i+1} = cn are known now
     const int n = par + 2 * i;
-    T y = (c1 * m.td[n] + cn * m.tu[n]) + c2 * m.tl[n];  // c2 = 0 in row 0
-    y = fma(y, sc, i == 0 ? ta : (T)0);
-    put(i, y);
+    const T y = (c1 * m.td[n] + cn * m.tu[n]) + c2 * m.tl[n];  // c2 = 0 in row 0
+    put(i, y + (i == 0 ? ta : (T)0));
     c2 = c1;
     c1 = cn;
   };
-  double c0, a;
-  auto boundary = [&](double s1) {
-    const double rh = fma(-s1, U, widen<T>(r0));
-    c0 = fma(g, ck, rh * cb);
-    a = fma(g, cd, -(rh * cc));
-    ta = narrow<T>(a);
-  };
-  if constexpr (sizeof(T) == 4) {
-    const float* rr = reinterpret_cast<const float*>(slab) + lane;
-    long long* sw = reinterpret_cast<long long*>(slab) + lane;  // overwrites right-hand sides already used
-    long long s = 0;
-    const int ex = ((__float_as_int(mx) >> 23) & 0xff) + 1;  // mx < 2^(ex - 127)
-    int top = 0;
-    rows_ahead<4, -1, int2>(v, il, 1, fv, [&](int i, int2 f) {
-      s = fx_from(rr[i * 32], ex) + fx_mul(s, f);
-      __syncwarp();
-      sw[i * 32] = s;
-      const int h = (int)(s >> 32);
-      top = max(top, h ^ (h >> 31));
-    });
-    boundary(ldexp_small(__ll2double_rn(s), ex - 127 - 55));
-    // range of the substitution: both |s| and |c_0| below 2^(e3 - 127); up to 64 rows of s and 2 c_0 (|t| < 1
-    // but in the row under n = 0, where it is below 2) then stay below 2^62.  The scales are powers of
-    // two, so moving s from its own to this one is a shift.
-    const int e0 = (int)((__double2hiint(c0) >> 20) & 0x7ff) - 895;
-    const int es = ex - 55 + (32 - __clz(top)) + 32;
-    const int e3 = max(max(es, e0), 1);
-    const int sh = e3 - ex, shr = min(max(sh, 0), 63), shl = max(-sh, 0);
-    long long c = __double2ll_rn(ldexp_small(c0, 55 - (e3 - 127)));
-    sc = __int_as_float(min(e3, 254) << 23);
-    c1 = fx_float(c);
-    rows_ahead<4, 1, int2>(t, 1, il, ft, [&](int i, int2 f) {
-      c = ((sw[i * 32] << shl) >> shr) + fx_mul(c, f);
-      row(i - 1, fx_float(c));
-    });
-  } else {
-    double* sw = reinterpret_cast<double*>(slab) + lane;
-    double s = 0.0;
-    rows_ahead<4, -1, int2>(v, il, 1, fv, [&](int i, int2 f) {
-      s = fma(as_double(f), s, sw[i * 32]);
-      sw[i * 32] = s;
-    });
-    boundary(s);
-    double c = c0;
-    c1 = c0;
-    rows_ahead<4, 1, int2>(t, 1, il, ft, [&](int i, int2 f) {
-      c = fma(as_double(f), c, sw[i * 32]);
-      row(i - 1, c);
-    });
-  }
+  double c = c0;
+  rows_ahead<4, 1, double>(t, 1, il, ft, [&](int i, double f) {
+    c = fma(f, c, sw[i * 32]);
+    row(i - 1, narrow<T>(c));
+  });
   row(il, (T)0);
   if (SLIP) {
     qd = fma(c0, w0d, qd);
@@ -470,18 +394,16 @@ __global__ void __launch_bounds__(kSolveThreads, 2) solve_tile_kernel(const __gr
     }
     m.ki[(t & 15) * kSolveK + kc] = e;
   };
-  // float plans substitute in units of 2^-55
-  const T unit = sizeof(T) == 4 ? (T)2.7755575615628914e-17 : (T)1;
   for (int i = threadIdx.x; i < N; i += kSolveThreads) {
-    m.tl[i] = bandT[i] * unit;
-    m.td[i] = bandT[N + i] * unit;
-    m.tu[i] = bandT[2 * N + i] * unit;
+    m.tl[i] = bandT[i];
+    m.td[i] = bandT[N + i];
+    m.tu[i] = bandT[2 * N + i];
   }
   if (wi < kGroup / 2) entry(2 * wi);
   const T tsH = (T)g.sH, tie = (T)g.inv_eta;
   const int par = wi & 1;
   const int il = (N - 1 - par) >> 1;  // last row index of this parity
-  unsigned char* slab = reinterpret_cast<unsigned char*>(m.sw + (size_t)wi * solve_rows(N) * 32);
+  double* slab = m.sw + (size_t)wi * solve_rows(N) * 32;
   const double* edge = tab.edge + (size_t)par * 7 * KP;
 
   for (int s = 0; s < nt + 2; ++s) {
@@ -521,9 +443,8 @@ __global__ void __launch_bounds__(kSolveThreads, 2) solve_tile_kernel(const __gr
       hb += 2 * (no_h ? il - 1 : il) * rs;
       T dh = (T)0;  // derivative recurrence of h over the opposite parity
       double ga = 0.0, q = 0.0, qd = 0.0;
-      T mx;
       functionals<T, false, In>(
-          il, tb, slab, lane, ga, q, qd, mx,
+          il, tb, slab, lane, ga, q, qd,
           [&](In& x, bool more) {
             x.f = fb[0];
             x.q = fb[fs];
@@ -543,7 +464,7 @@ __global__ void __launch_bounds__(kSolveThreads, 2) solve_tile_kernel(const __gr
       if (par == 0) dh = dh * (T)0.5;
       T* po = m.p + (size_t)(s & 1) * N * 32 + par * 32 + lane;
       m.pv[((s & 1) * 2 + par) * 32 + lane] =
-          sweeps<T, false>(il, par, tb, edge + kp, slab, lane, m, mx, sx * f0 + sy * q0 + tsH * dh, ga, q, qd,
+          sweeps<T, false>(il, par, tb, edge + kp, slab, lane, m, sx * f0 + sy * q0 + tsH * dh, ga, q, qd,
                            [&](int i, T y) {
                              po[i * 64] = y;
                            });
@@ -559,7 +480,6 @@ __global__ void __launch_bounds__(kSolveThreads, 2) solve_tile_kernel(const __gr
       T* const y0 = reinterpret_cast<T*>(kbuf + (size_t)f * N * K + kid) + part + par * rs;
       const T v0 = __ldcs(y0);
       double ga, q = 0.0, qd = 0.0;
-      T mx;
       const T* yb = y0 + 2 * il * rs;
       T r0;
       if (f < 2) {
@@ -570,7 +490,7 @@ __global__ void __launch_bounds__(kSolveThreads, 2) solve_tile_kernel(const __gr
         const T sk = part ? (T)kf : -(T)kf;
         const T* po = pi + par * 32 + (lane ^ 16);
         functionals<T, SLIP, T>(
-            il, tb, slab, lane, ga, q, qd, mx,
+            il, tb, slab, lane, ga, q, qd,
             [&](T& x, bool more) {
               x = __ldcs(yb);
               if (more) yb -= 2 * rs;
@@ -586,7 +506,7 @@ __global__ void __launch_bounds__(kSolveThreads, 2) solve_tile_kernel(const __gr
           if (n + 1 < N) dp = dp + po[i * 64] * (T)(2 * (n + 1));
         };
         functionals<T, false, T>(
-            il, tb, slab, lane, ga, q, qd, mx,
+            il, tb, slab, lane, ga, q, qd,
             [&](T& x, bool more) {
               x = __ldcs(yb);
               if (more) yb -= 2 * rs;
@@ -602,7 +522,7 @@ __global__ void __launch_bounds__(kSolveThreads, 2) solve_tile_kernel(const __gr
       const bool keep = e.kid > 0;  // not beyond the end, not k = 0
       T* yo = y0;
       const int slot = t % kVRing;
-      const double vw = sweeps<T, SLIP>(il, par, tb, edge + kp, slab, lane, m, mx, r0, ga, q, qd, [&](int, T y) {
+      const double vw = sweeps<T, SLIP>(il, par, tb, edge + kp, slab, lane, m, r0, ga, q, qd, [&](int, T y) {
         if (keep) __stcs(yo, y);
         yo += 2 * rs;
       });
@@ -634,11 +554,6 @@ __global__ void solve_table_kernel(Geometry g, const double* __restrict__ band, 
   const double kx = 2.0 * M_PI * (double)kxi / g.Lx, ky = 2.0 * M_PI * (double)kyi / g.Ly;
   const double kk = sqrt(kx * kx + ky * ky), kap = kk * kk;
   const double sH = 2.0 / g.H, sig = sH * sH;
-  auto store = [](double v) {
-    if (sizeof(T) == 8) return make_int2(__double2loint(-v), __double2hiint(-v));
-    const long long f = __double2ll_rn(-v * 1152921504606846976.0);  // 2^60
-    return make_int2((int)f, (int)((f + 0x80000000ll) >> 32));
-  };
   for (int par = 0; par < 2; ++par) {
     const int nlast = ((N - 1 - par) & 1) ? N - 2 : N - 1;
     double t_next = 0.0, b = sH * bP[nlast] + kk * bQ[nlast], w = 0.0, wd = 0.0;
@@ -651,8 +566,8 @@ __global__ void solve_table_kernel(Geometry g, const double* __restrict__ band, 
       wd = bP[n] - t_next * wd;
       tab.gw[o] = make_double2(b, w);
       if (tab.wd) tab.wd[o] = wd;
-      tab.V[o] = make_int2(__double2loint(U * rho), __double2hiint(U * rho));
-      tab.t[o] = store(t);
+      tab.V[o] = U * rho;
+      tab.t[o] = -t;
       tab.rho[o] = (T)rho;
       b = (sH * bP[n - 2] + kk * bQ[n - 2]) - b * t;
       t_next = t;
@@ -679,8 +594,8 @@ __global__ void solve_table_kernel(Geometry g, const double* __restrict__ band, 
         od = tab.wd[o] - V * od;
         tab.wd[o] = od;
       }
-      V = as_double(tab.V[o]);
-      tab.V[o] = store(V);
+      V = tab.V[o];
+      tab.V[o] = -V;
     }
   }
 }

@@ -3,6 +3,7 @@ of unequal length, rows short of whole batches), boxes whose wavenumbers end ins
 tiles than a block, odd sizes without Nyquist columns, and the first node count past it; each against
 the oracle at the parity bars (1e-9 in double, 1e-5 in mixed precision)."""
 
+import numpy as np
 import pytest
 
 from oracle.stokes import mobility
@@ -52,3 +53,16 @@ def test_one_block_runs_all_tiles_and_the_zero_mode(nx, ny, nz, zmax, precision)
     assert rel_l2(U0, U_ref) <= TOL[precision]
     assert rel_l2(W0, W_ref) <= TOL[precision]
     assert (U1 == U0).all() and (W1 == W0).all()
+
+
+@pytest.mark.parametrize("nz", [33, 97])
+@pytest.mark.parametrize("torque", [True, False])
+def test_overflow_is_never_a_finite_wrong_number(nz, torque):
+    """Forces of 1e37 overflow the float spectra: what comes out is not finite, or right at the parity bar."""
+    params = small_params("slit", nx=40, ny=36, nz=nz, zmax=8.0, torque=torque)
+    pos, F, T = random_particles(params, 20, seed=3, torques=torque)
+    T = None if T is None else 0.0 * T
+    U_ref, _ = mobility(oracle_params(params), pos, F, T)
+    U, _ = gpu_mobility(params, pos, 1e37 * F, T, "mixed")
+    finite = np.isfinite(U)
+    assert np.all(np.abs(U[finite] / 1e37 - U_ref[finite]) <= TOL["mixed"] * np.abs(U_ref).max())
