@@ -178,10 +178,17 @@ struct Server {
     const int64_t blocks = std::min<int64_t>(152 * 4, (K + kBvpThreads - 1) / kBvpThreads);
     int64_t b = nf * nz * ny * pitch * 2 * ts;                          // grid
     b += nmax * (rec + 8 + 15 * 8) + 3 * nbins * 4;                      // records, bins, staging
-    // solve workspace (the tiled solve, which takes none, applies to every column up to one pass of blocks)
-    if (nz > 128 || blocks >= 152 * 3) b += blocks * kBvpThreads * nz * (3 * 16 + 3 * 8 + 2 * ts);
+    Geometry g;  // what the solve's rule looks at
+    memset(&g, 0, sizeof(g));
+    g.nkx = (int)nkx; g.ny = (int)ny; g.nz = (int)nz; g.mode = r.wall_mode;
+    for (double x : {r.walls.slip_bottom, r.walls.slip_top, r.walls.uw_bottom[0], r.walls.uw_bottom[1],
+                     r.walls.uw_top[0], r.walls.uw_top[1]})
+      g.slip = g.slip || x != 0.0;
+    if (solve_tile_applies(g, r.kp.precision))  // the tiled solve's table; else workspace and factorisation table
+      b += (int64_t)solve_tile_table_bytes(g, r.kp.precision);
+    else
+      b += blocks * kBvpThreads * nz * (3 * 16 + 3 * 8 + 2 * ts) + nkx * (ny / 2 + 1) * nz * 4 * 8;
     b += 3 * nz * K * 2 * ts + 12 * K * 2 * ts;                          // kbuf, kaux
-    b += nkx * (ny / 2 + 1) * (nz * 48 + 14 * 8);                        // the solve's table
     if (ts == 8) b += nkx * (ny / 2 + 1) * nz * 16 + 256 * nz * nz;      // the folded transforms' tables
     // partial sums of the tile-gather interpolation (forces only, or equal supports with the
     // spectral curl): slots of the tiles a support can overlap x fields x particles

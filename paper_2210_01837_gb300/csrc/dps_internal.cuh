@@ -292,9 +292,10 @@ template <typename T> int bvp_prepare(Plan& p);
 // the factorisation table of the FP64 solve (allocated and filled at plan creation); DPS_ERR_OOM
 // leaves the plan on the factorise-as-you-go solve
 dps_status bvp_factor_table(Plan& p);
-// the tiled solve (solve.cu): where it applies, its resident grid (0 on a CUDA error), its table (allocated
-// and filled; as bvp_factor_table), and its launcher
+// the tiled solve (solve.cu): where it applies (from nkx, ny, nz, slip and mode), its resident grid (0 on a CUDA
+// error), its table (bytes; allocated and filled, as bvp_factor_table), and its launcher
 bool solve_tile_applies(const Geometry& g, int precision);
+size_t solve_tile_table_bytes(const Geometry& g, int precision);
 template <typename T> int solve_tile_prepare(const Plan& p);
 dps_status solve_tile_table(Plan& p);
 template <typename T> void launch_solve_tile(const Plan& p, int kx0, int w, cudaStream_t s);

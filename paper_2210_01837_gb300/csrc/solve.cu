@@ -27,6 +27,7 @@ namespace {
 constexpr int kSolveK = 16;       // wavenumbers per tile
 constexpr int kSolveWarps = 8;    // 3 velocity components + pressure, two parities each
 constexpr int kSolveThreads = 32 * kSolveWarps;
+constexpr size_t kMaxBlockSmem = 227 * 1024;  // shared memory a block can have
 // wavenumber constants and wall amplitudes are long serial chains on the FP64 pipe (a square root; up to
 // divisions and an exponential): they are done for 8 tiles at a time, two tiles a warp, one warp on each
 // sub-partition, so that they hold up one step in eight
@@ -607,11 +608,12 @@ __global__ void solve_table_kernel(Geometry g, const double* __restrict__ band, 
 // an SM to cover its own latencies (up to 72 nodes in float; 384 x 384 x 97 alone gains 8 %, but a batch of
 // systems with such columns, which fill the GPU together, loses 4 %), and columns long enough to outweigh
 // a tile's fixed part: at 19 nodes and 3.6 million wavenumbers it takes 7.5 ms against 6.0, at 33 to 65
-// nodes it wins at every size measured.
+// nodes it wins at every size measured.  In every case a block has to fit: in double with wall conditions,
+// whose derivatives take 9 KB more, 127 and 128 nodes do not.
 template <typename T>
 bool solve_tile_applies_t(const Geometry& g) {
   const int64_t one_pass = 152 * 3 * kBvpThreads;
-  if (g.nz > 128) return false;
+  if (g.nz > 128 || solve_smem_bytes<T>(g.nz, g.slip != 0) > kMaxBlockSmem) return false;
   return (int64_t)g.nkx * g.ny <= one_pass ||
          (g.nz >= 25 && 2 * (solve_smem_bytes<T>(g.nz, g.slip != 0) + 1024) <= 228 * 1024);
 }
@@ -626,17 +628,22 @@ int solve_tile_prepare(const Plan& p) {
   int per_sm = 0, sms = 0;
   const size_t b = solve_smem_bytes<T>(p.g.nz, p.g.slip != 0);
   const void* k = p.g.slip ? (const void*)solve_tile_kernel<T, true> : (const void*)solve_tile_kernel<T, false>;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kSolveThreads, b) != cudaSuccess) return 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kSolveThreads, b) != cudaSuccess || per_sm < 1) return 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device) != cudaSuccess) return 0;
   const int64_t tiles = ((int64_t)p.g.nkx * p.g.ny + kSolveK - 1) / kSolveK;
-  const int64_t most = (int64_t)(per_sm < 1 ? 1 : per_sm) * sms;
+  const int64_t most = (int64_t)per_sm * sms;
   return (int)(tiles < most ? tiles : most);
+}
+
+size_t solve_tile_table_bytes(const Geometry& g, int precision) {
+  const int64_t KP = (int64_t)g.nkx * (g.ny / 2 + 1);
+  return precision == DPS_MIXED ? solve_table_bytes<float>(g, KP) : solve_table_bytes<double>(g, KP);
 }
 
 dps_status solve_tile_table(Plan& p) {
   const int64_t KP = (int64_t)p.g.nkx * (p.g.ny / 2 + 1);
   const bool mixed = p.precision == DPS_MIXED;
-  const size_t bytes = mixed ? solve_table_bytes<float>(p.g, KP) : solve_table_bytes<double>(p.g, KP);
+  const size_t bytes = solve_tile_table_bytes(p.g, p.precision);
   void* q = nullptr;
   if (cudaMalloc(&q, bytes) != cudaSuccess) {
     cudaGetLastError();

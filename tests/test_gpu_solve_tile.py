@@ -66,3 +66,18 @@ def test_overflow_is_never_a_finite_wrong_number(nz, torque):
     U, _ = gpu_mobility(params, pos, 1e37 * F, T, "mixed")
     finite = np.isfinite(U)
     assert np.all(np.abs(U[finite] / 1e37 - U_ref[finite]) <= TOL["mixed"] * np.abs(U_ref).max())
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("mode", ["bottom_wall", "slit"])
+@pytest.mark.parametrize("nx,ny,nz,zmax", SHAPES + [(16, 12, 126, 6.0), (16, 12, 127, 6.0)])
+def test_wall_conditions_at_the_edges_match_oracle(nx, ny, nz, zmax, mode, precision):
+    """Slip and wall velocities take more shared memory and a longer table row: the last node counts whose
+    block fits (126 in double) and the first that take the thread-per-wavenumber solve."""
+    params = small_params(mode, nx=nx, ny=ny, nz=nz, zmax=zmax, torque=True)
+    params.update({k: v for k, v in WALLS.items() if mode == "slit" or k.endswith("bottom")})
+    pos, F, T = random_particles(params, 7, seed=nz)
+    U_ref, W_ref = mobility(oracle_params(params), pos, F, T)
+    U, W = gpu_mobility(params, pos, F, T, precision)
+    assert rel_l2(U, U_ref) <= TOL[precision]
+    assert rel_l2(W, W_ref) <= TOL[precision]
