@@ -603,19 +603,27 @@ __global__ void solve_table_kernel(Geometry g, const double* __restrict__ band, 
 
 }  // namespace
 
-// Up to one pass of the thread-per-wavenumber solve's grid, that solve's time is the latency of one thread's
-// serial rows and this one wins at any length (120 x 120 x 33: 155 -> 47 us).  Beyond, it needs two blocks
-// an SM to cover its own latencies (up to 72 nodes in float; 384 x 384 x 97 alone gains 8 %, but a batch of
-// systems with such columns, which fill the GPU together, loses 4 %), and columns long enough to outweigh
-// a tile's fixed part: at 19 nodes and 3.6 million wavenumbers it takes 7.5 ms against 6.0, at 33 to 65
-// nodes it wins at every size measured.  In every case a block has to fit: in double with wall conditions,
-// whose derivatives take 9 KB more, 127 and 128 nodes do not.
+// Where it is the faster one.  P: wavenumbers in passes of the thread-per-wavenumber solve's grid; figures are
+// that solve's time over this one's, without walls / with (whose amplitudes lengthen its one thread's chain).
+//  - Up to one pass the other solve waits on the latency of one thread's serial rows: 120 x 120 x 33 155 -> 47 us.
+//    Where two blocks fit an SM (up to 70 nodes in float) this one wins at every size but the fullest pass:
+//    33 nodes, P = 0.14 2.7 / 3.4, 0.57 1.3 / 1.8, 0.97 1.04 / 1.4; 33 in double 2.1 / 2.7, 1.07 / 1.3, 0.94 / 1.08.
+//    Where only one fits, it covers less of its own latencies: 97 nodes, P = 0.28 1.46 / 2.2, 0.5 1.02 / 1.6,
+//    0.57 0.86 / 1.3, 0.88 0.70 / 1.03; in double 1.3 / 1.7, 1.03 / 1.3, 0.88 / 1.14, 0.87 / 1.02.
+//  - Beyond, it needs two blocks an SM (97 nodes, P = 5 0.72 / 0.78) and columns long enough to outweigh a tile's
+//    fixed part.  Float from 33 nodes on wins at every size (P = 1.27 1.34 / 1.6, 5 1.15 / 1.16, 81 1.03 / 1.01).
+//    Shorter columns and double win by the other's last pass while that counts: 25 nodes, P = 1.27 1.25 / 1.5,
+//    5 1.06 / 1.07, 7 0.97 / 0.97, 81 0.94 / 0.94; 33 in double 1.2 / 1.3, 1.02 / 1.05, 0.97 / 0.97.
+// In every case a block has to fit: in double with wall conditions, whose derivatives take 9 KB more, 127 and
+// 128 nodes do not.
 template <typename T>
 bool solve_tile_applies_t(const Geometry& g) {
-  const int64_t one_pass = 152 * 3 * kBvpThreads;
-  if (g.nz > 128 || solve_smem_bytes<T>(g.nz, g.slip != 0) > kMaxBlockSmem) return false;
-  return (int64_t)g.nkx * g.ny <= one_pass ||
-         (g.nz >= 25 && 2 * (solve_smem_bytes<T>(g.nz, g.slip != 0) + 1024) <= 228 * 1024);
+  const size_t b = solve_smem_bytes<T>(g.nz, g.slip != 0);
+  if (g.nz > 128 || b > kMaxBlockSmem) return false;
+  const bool two = 2 * (b + 1024) <= 228 * 1024;
+  const double passes = (double)g.nkx * g.ny / (152.0 * 3 * kBvpThreads);
+  if (passes <= 1.0) return two || passes <= (g.mode == DPS_FREE ? 0.5 : 0.9);
+  return two && g.nz >= 25 && ((sizeof(T) == 4 && g.nz >= 33) || passes <= 6.0);
 }
 
 bool solve_tile_applies(const Geometry& g, int precision) {

@@ -81,3 +81,32 @@ def test_wall_conditions_at_the_edges_match_oracle(nx, ny, nz, zmax, mode, preci
     U, W = gpu_mobility(params, pos, F, T, precision)
     assert rel_l2(U, U_ref) <= TOL[precision]
     assert rel_l2(W, W_ref) <= TOL[precision]
+
+
+# (mode, precision, nx, ny, nz, tiled): either side of the lines of the rule
+ROUTES = [("free", "mixed", 240, 240, 81, True), ("free", "mixed", 256, 240, 81, False),
+          ("free", "fp64", 240, 240, 66, True), ("free", "fp64", 256, 240, 66, False),
+          ("slit", "mixed", 320, 320, 81, True), ("slit", "mixed", 324, 324, 81, False),
+          ("bottom_wall", "fp64", 320, 320, 66, True), ("bottom_wall", "fp64", 324, 324, 66, False),
+          ("free", "mixed", 336, 336, 65, True), ("slit", "mixed", 384, 384, 24, False),
+          ("slit", "mixed", 384, 384, 25, True), ("bottom_wall", "mixed", 840, 840, 32, False),
+          ("bottom_wall", "mixed", 840, 840, 33, True), ("free", "fp64", 840, 840, 33, False),
+          ("free", "fp64", 800, 800, 33, True)]
+
+
+@pytest.mark.parametrize("mode,precision,nx,ny,nz,tiled", ROUTES)
+def test_either_side_of_the_rule_matches_the_general_solve(mode, precision, nx, ny, nz, tiled, monkeypatch):
+    """The chosen solve against the one that factorises as it goes and takes every plan; which one was
+    chosen shows in the grid (one block of 128 wavenumbers each, or fewer tiles' blocks)."""
+    params = small_params(mode, nx=nx, ny=ny, nz=nz, zmax=7.0, torque=False)
+    pos, F, _ = random_particles(params, 40, seed=nz, torques=False)
+    plan = binding.Plan.from_params(params, with_torque=False, precision=precision, max_n=len(pos))
+    blocks = plan.info().solve_blocks
+    U, _ = gpu_mobility(params, pos, F, None, precision, plan=plan)
+    plan.close()
+    monkeypatch.setenv("DPS_SOLVE_TABLE", "0")
+    general = binding.Plan.from_params(params, with_torque=False, precision=precision, max_n=len(pos))
+    assert (blocks < general.info().solve_blocks) == tiled
+    U_ref, _ = gpu_mobility(params, pos, F, None, precision, plan=general)
+    general.close()
+    assert rel_l2(U, U_ref) <= TOL[precision]
