@@ -119,8 +119,9 @@ template <typename T, int NB>
 __global__ void __launch_bounds__(kBvpThreads) fwd_kernel(Geometry g, const T* __restrict__ ct_g,
                                                           const T* __restrict__ dct_g, int npad, int smem_tabs,
                                                           const cplx<T>* __restrict__ grid, cplx<T>* __restrict__ kbuf,
-                                                          const int* __restrict__ zrange, int kx0, int w) {
+                                                          const int* __restrict__ zrange, int kx0, int w, int thin) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  if (thin > 0 && zrange[1] - zrange[0] >= thin) return;  // the folded transform's turn
   const int N = g.nz;
   T* sm = reinterpret_cast<T*>(smraw);
   const T* Ct = stage_table<T>(sm, ct_g, N * npad, smem_tabs != 0);
@@ -944,8 +945,9 @@ __global__ void __launch_bounds__(kBvpThreads) bwd_kernel(Geometry g, const T* _
                                                           const T* __restrict__ zeta_g, int cpad, int smem_tabs,
                                                           const cplx<T>* __restrict__ kbuf,
                                                           const cplx<T>* __restrict__ kaux, cplx<T>* __restrict__ grid,
-                                                          const int* __restrict__ zrange, int kx0, int w) {
+                                                          const int* __restrict__ zrange, int kx0, int w, int thin) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  if (thin > 0 && zrange[1] - zrange[0] >= thin) return;  // the folded transform's turn
   const int N = g.nz;
   T* sm = reinterpret_cast<T*>(smraw);
   const int tab = N * cpad;
@@ -1126,9 +1128,10 @@ __global__ void __launch_bounds__(MB == 3 ? kFwdCompactThreads : fwd_max_threads
                                                                         const cplx<T>* __restrict__ grid,
                                                                         cplx<T>* __restrict__ kbuf,
                                                                         const int* __restrict__ zrange, int kx0, int w,
-                                                                        int cz) {
+                                                                        int cz, int thin) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ KTile kt;
+  if (thin > 0 && zrange[1] - zrange[0] >= thin) return;  // the folded transform's turn
   constexpr int NF = TQ ? 6 : 3;  // staged fields per (plane, wavenumber); the first 3 (5) become a (a, b)
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int nthreads = blockDim.x;
@@ -1254,9 +1257,10 @@ __global__ void __launch_bounds__(32 * bwd_warps<T>(), sizeof(T) == 4 ? 3 : 1) b
                                                         int cpad, const T* __restrict__ zeta_g,
                                                         const cplx<T>* __restrict__ kbuf,
                                                         const cplx<T>* __restrict__ kaux, cplx<T>* __restrict__ grid,
-                                                        const int* __restrict__ zrange, int kx0, int w) {
+                                                        const int* __restrict__ zrange, int kx0, int w, int thin) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ KTile kt;
+  if (thin > 0 && zrange[1] - zrange[0] >= thin) return;  // the folded transform's turn
   constexpr bool DE = CURL && CORR > 0;              // derivative of the correction
   constexpr int NT = CURL ? (CORR > 0 ? 3 : 2) : 1;  // staged tables: IC, ICD, SD
   constexpr int NW = bwd_warps<T>();
@@ -1487,14 +1491,14 @@ size_t bwd_lane_smem(const Geometry& g) {
 }
 
 template <typename T, bool CURL, int CORR>
-void launch_bwd_lane(const Plan& p, int kx0, int w, cudaStream_t s) {
+void launch_bwd_lane(const Plan& p, int kx0, int w, int thin, cudaStream_t s) {
   const Geometry& g = p.g;
   const unsigned blocks = (unsigned)(((int64_t)w * g.ny + kLaneK - 1) / kLaneK);
   bwd_lane_kernel<T, bwd_pg<T>(), CURL, CORR><<<blocks, 32 * bwd_warps<T>(), bwd_lane_smem<T>(g), s>>>(
       g, reinterpret_cast<const T*>(p.kt.ict), reinterpret_cast<const T*>(p.kt.icdt),
       reinterpret_cast<const T*>(p.kt.sdt), p.kt.cpad, reinterpret_cast<const T*>(p.tab.zeta),
       reinterpret_cast<const cplx<T>*>(p.kt.kbuf), reinterpret_cast<const cplx<T>*>(p.kt.kaux),
-      reinterpret_cast<cplx<T>*>(p.grid), p.zrange, kx0, w);
+      reinterpret_cast<cplx<T>*>(p.grid), p.zrange, kx0, w, thin);
 }
 
 template <typename T, bool CURL, int CORR>
@@ -1560,9 +1564,14 @@ void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s) {
   cplx<T>* kbuf = reinterpret_cast<cplx<T>*>(p.kt.kbuf);
   cplx<T>* kaux = reinterpret_cast<cplx<T>*>(p.kt.kaux);
   const LaneCfg fc = fwd_lane_cfg<T>(g);
+  // beside the folded transforms: the dense ones for at most `thin` occupied planes (0: they take every call)
+  int thin = 0;
   if (part != 1 && p.cheb_fold) {
-    launch_cheb_fold(p, part == 2, kx0, w, s);
-  } else if (part != 1 && (p.cheb_columns & (part == 2 ? 2 : 1)) && (part == 2 || p.inject != 1)) {
+    thin = p.fold_thin[part == 2];
+    if (thin < g.nz) launch_cheb_fold(p, part == 2, kx0, w, s);
+    if (thin == 0) return;
+  }
+  if (part != 1 && (p.cheb_columns & (part == 2 ? 2 : 1)) && (part == 2 || p.inject != 1)) {
     launch_cheb_columns(p, part == 2, kx0, w, s);
   } else if (part == 0 && sizeof(T) == 4 && p.cheb_tc) {
     launch_cheb_fwd_tc(p, kx0, w, s);
@@ -1577,7 +1586,7 @@ void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s) {
       // is (70 registers) and measured slower compact (5.20 -> 5.30 ms on rollers_1m)
       if (fc.pg == PG && fc.threads <= kFwdCompactThreads && g.spectral_curl) {
         fwd_lane_kernel<T, PG, true, 3><<<lb, fc.threads, fc.smem, s>>>(g, ct, dct, p.kt.npad, grid, kbuf, p.zrange,
-                                                                        kx0, w, fc.cz);
+                                                                        kx0, w, fc.cz, thin);
         done = true;
       }
     }
@@ -1585,35 +1594,35 @@ void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s) {
     } else if (fc.pg == PG) {
       if (g.spectral_curl)
         fwd_lane_kernel<T, PG, true><<<lb, fc.threads, fc.smem, s>>>(g, ct, dct, p.kt.npad, grid, kbuf, p.zrange, kx0,
-                                                                     w, fc.cz);
+                                                                     w, fc.cz, thin);
       else
         fwd_lane_kernel<T, PG, false><<<lb, fc.threads, fc.smem, s>>>(g, ct, dct, p.kt.npad, grid, kbuf, p.zrange, kx0,
-                                                                      w, fc.cz);
+                                                                      w, fc.cz, thin);
     } else {
       if (g.spectral_curl)
         fwd_lane_kernel<T, PW, true><<<lb, fc.threads, fc.smem, s>>>(g, ct, dct, p.kt.npad, grid, kbuf, p.zrange, kx0,
-                                                                     w, fc.cz);
+                                                                     w, fc.cz, thin);
       else
         fwd_lane_kernel<T, PW, false><<<lb, fc.threads, fc.smem, s>>>(g, ct, dct, p.kt.npad, grid, kbuf, p.zrange, kx0,
-                                                                      w, fc.cz);
+                                                                      w, fc.cz, thin);
     }
   } else if (part == 2 && sizeof(T) == 4 && p.cheb_tc_bwd) {
     launch_cheb_bwd_tc(p, kx0, w, s);
   } else if (part == 2 && bwd_lane_smem<T>(g) > 0) {
     const int corr = g.mode == DPS_FREE ? 0 : (g.mode == DPS_SLIT ? 2 : 1);
     if (g.spectral_curl) {
-      if (corr == 0) launch_bwd_lane<T, true, 0>(p, kx0, w, s);
-      else if (corr == 1) launch_bwd_lane<T, true, 1>(p, kx0, w, s);
-      else launch_bwd_lane<T, true, 2>(p, kx0, w, s);
+      if (corr == 0) launch_bwd_lane<T, true, 0>(p, kx0, w, thin, s);
+      else if (corr == 1) launch_bwd_lane<T, true, 1>(p, kx0, w, thin, s);
+      else launch_bwd_lane<T, true, 2>(p, kx0, w, thin, s);
     } else {
-      if (corr == 0) launch_bwd_lane<T, false, 0>(p, kx0, w, s);
-      else if (corr == 1) launch_bwd_lane<T, false, 1>(p, kx0, w, s);
-      else launch_bwd_lane<T, false, 2>(p, kx0, w, s);
+      if (corr == 0) launch_bwd_lane<T, false, 0>(p, kx0, w, thin, s);
+      else if (corr == 1) launch_bwd_lane<T, false, 1>(p, kx0, w, thin, s);
+      else launch_bwd_lane<T, false, 2>(p, kx0, w, thin, s);
     }
   } else if (part == 0) {
     fwd_kernel<T, NB><<<blocks, kBvpThreads, p.kt.fwd_smem, s>>>(
         g, reinterpret_cast<const T*>(p.kt.ct), reinterpret_cast<const T*>(p.kt.dct), p.kt.npad, p.kt.fwd_smem > 0,
-        grid, kbuf, p.zrange, kx0, w);
+        grid, kbuf, p.zrange, kx0, w, thin);
   } else if (part == 1 && p.solve_tile) {
     launch_solve_tile<T>(p, kx0, w, s);
   } else if (part == 1) {
@@ -1641,11 +1650,11 @@ void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s) {
     bwd_kernel<T, CB, true><<<blocks, kBvpThreads, p.kt.bwd_smem, s>>>(
         g, reinterpret_cast<const T*>(p.kt.ict), reinterpret_cast<const T*>(p.kt.icdt),
         reinterpret_cast<const T*>(p.kt.sdt), reinterpret_cast<const T*>(p.tab.zeta), p.kt.cpad, p.kt.bwd_smem > 0, kbuf,
-        kaux, grid, p.zrange, kx0, w);
+        kaux, grid, p.zrange, kx0, w, thin);
   } else {
     bwd_kernel<T, CB, false><<<blocks, kBvpThreads, p.kt.bwd_smem, s>>>(
         g, reinterpret_cast<const T*>(p.kt.ict), nullptr, nullptr, reinterpret_cast<const T*>(p.tab.zeta), p.kt.cpad,
-        p.kt.bwd_smem > 0, kbuf, kaux, grid, p.zrange, kx0, w);
+        p.kt.bwd_smem > 0, kbuf, kaux, grid, p.zrange, kx0, w, thin);
   }
 }
 

@@ -210,8 +210,9 @@ __global__ void __launch_bounds__((TQ ? 20 : 12) * 32) fold_fwd_kernel(const __g
                                                                       const cplx<T>* __restrict__ grid,
                                                                       cplx<T>* __restrict__ kbuf,
                                                                       const int* __restrict__ zrange, int kx0, int w,
-                                                                      double hx, double hy) {
+                                                                      double hx, double hy, int thin) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  if (thin > 0 && zrange[1] - zrange[0] < thin) return;  // the dense transform's turn
   constexpr int NF = TQ ? 5 : 3, NW = 4 * NF;
   const int N = g.nz, M = (N - 1) / 2;
   T* sx = reinterpret_cast<T*>(smraw);  // [NF][N][32]
@@ -308,8 +309,9 @@ __global__ void __launch_bounds__((CURL ? 20 : 12) * 32) fold_bwd_kernel(const _
                                                                         const cplx<T>* __restrict__ kaux,
                                                                         cplx<T>* __restrict__ grid,
                                                                         const int* __restrict__ zrange, int kx0, int w,
-                                                                        double hx, double hy) {
+                                                                        double hx, double hy, int thin) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  if (thin > 0 && zrange[1] - zrange[0] < thin) return;  // the dense transform's turn
   constexpr int NF = CURL ? 5 : 3, NW = 4 * NF;
   const int N = g.nz, M = (N - 1) / 2;
   T* sx = reinterpret_cast<T*>(smraw);  // [NF][N][32]
@@ -468,6 +470,28 @@ bool cheb_fold_applies(const Plan& p) {
   return p.precision == DPS_FP64 && (g.nz - 1) % 8 == 0 && g.nz >= 9 && g.nz <= 129;
 }
 
+// Folding transforms whole columns; the dense kernels only read (forward) or form (backward) the occupied
+// planes, whose number a call's particles decide on the device.  Where the dense ones can be the faster both are
+// launched, and each leaves at once when it is the other's turn.  The largest number of planes at which the
+// dense kernel is taken, from both over 17 to 129 nodes (dense over folded time at that number / at the next
+// measured one; 256 x 240, forces only, free space if not said):
+//   forward, any mode: 33 nodes 12: 0.95 / 1.1, 65 nodes 15: 0.93 / 1.04, 97 nodes 18: 0.98 / 1.10, 129 nodes
+//   21: 0.93 / 1.10; with torques it wins by 5 to 20 % there.  All 9 planes of 9 nodes: 0.7 with torques.
+//   backward: 33 nodes 8: 0.90 / 1.10, 65 nodes 16: 0.96 / 1.22, 97 nodes 16: 0.77 / 0.97, 121 nodes 24: 0.92 / 1.06,
+//   129 nodes 8: 0.61 / 0.85.  Walls and curls cost the dense kernel terms for all nodes: 65 nodes 1.07 and up
+//   with either; 97 nodes 0.83 with curl, 0.97 with walls, 1.09 with both; 121 nodes 16: bottom wall and curl 0.89,
+//   two walls and curl 1.04; 129 nodes (per-thread kernel) 0.39 to 0.96 at 8, in free space with curl 0.76 at 16.
+int fold_thin_planes(const Geometry& g, bool backward) {
+  const int N = g.nz;
+  if (!backward) return 9 + N / 10;
+  const bool walls = g.mode != DPS_FREE, curl = g.spectral_curl != 0;
+  if (N > 128) return !walls && curl ? 16 : 8;
+  if (N > 97) return !walls ? 24 : (g.mode == DPS_SLIT && curl ? 0 : 16);
+  if (N > 65) return walls && curl ? 0 : 16;
+  if (walls || curl) return 0;
+  return N > 33 ? 16 : 8;
+}
+
 size_t cheb_fold_bytes(const Geometry& g) {
   const size_t KP = (size_t)g.nkx * (g.ny / 2 + 1);
   return 2 * fold_table_values<double>(g.nz) * sizeof(double) + (g.mode != DPS_FREE ? KP * g.nz * sizeof(double2) : 0);
@@ -488,6 +512,7 @@ dps_status cheb_fold_prepare(Plan& p) {
     return DPS_ERR_OOM;
   }
   p.kt.fold = reinterpret_cast<double*>(q);
+  for (int d = 0; d < 2; ++d) p.fold_thin[d] = fold_thin_planes(g, d == 1);
   p.device_bytes += (int64_t)bytes;
   const std::vector<T> f = fold_table<T>(g.nz, 2.0 / (g.nz - 1)), b = fold_table<T>(g.nz, 1.0 / ((double)g.nx * (double)g.ny));
   if (cudaMemcpy(p.kt.fold, f.data(), nt * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -519,19 +544,20 @@ void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t
   const double2* ecf = g.mode != DPS_FREE ? reinterpret_cast<const double2*>(p.kt.fold + 2 * nt) : nullptr;
   const int64_t KP = (int64_t)g.nkx * (g.ny / 2 + 1);
   const double hx = M_PI / g.Lx, hy = M_PI / g.Ly;
+  const int thin = p.fold_thin[backward];
   fold_dispatch(fold_bucket(g.nz), [&](auto hp) {
     constexpr int HP = decltype(hp)::value;
     const int th = 32 * 4 * nf;
     if (!backward && g.spectral_curl)
-      fold_fwd_kernel<T, true, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy);
+      fold_fwd_kernel<T, true, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy, thin);
     else if (!backward)
-      fold_fwd_kernel<T, false, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy);
+      fold_fwd_kernel<T, false, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy, thin);
     else if (g.spectral_curl)
       fold_bwd_kernel<T, true, HP><<<blocks, th, smem, s>>>(g, p.kt.fold + nt, ecf, KP, kbuf, kaux, grid, p.zrange, kx0, w,
-                                                           hx, hy);
+                                                           hx, hy, thin);
     else
       fold_bwd_kernel<T, false, HP><<<blocks, th, smem, s>>>(g, p.kt.fold + nt, ecf, KP, kbuf, kaux, grid, p.zrange, kx0,
-                                                            w, hx, hy);
+                                                            w, hx, hy, thin);
   });
 }
 

@@ -165,6 +165,7 @@ struct Plan {
   int cheb_columns;     // three-field float transforms in registers: bit 0 forward, bit 1 backward
   int cheb_tc_bwd;      // backward Chebyshev transform on the tensor cores (spectral-curl torques)
   int cheb_fold;        // Chebyshev transforms by folding (double precision, nz - 1 a multiple of 8)
+  int fold_thin[2];     // forward, backward: most occupied planes at which the dense transforms run instead
   int cheb_tc_bwd_parts;  // launches of the backward transform (output planes split beyond 96 nodes)
   int cheb_tc_grid;     // persistent blocks of that kernel
   int inject;           // failure injection of the next apply (dpstokes_debug_inject)

@@ -666,10 +666,12 @@ dps_status dpstokes_plan_info(dps_plan_t plan, dps_plan_info* out) {
   out->alpha_D = p->g.with_torque ? p->g.kD.alpha : 0.0;
   // init, records, 3 binning, spread, x pass, 5 per column chunk, x pass, interpolation (+ its
   // finishing kernel for the tile gather)
-  // (+ the B-operand image kernel before each tensor-core transform)
+  // (+ the B-operand image kernel before each tensor-core transform, the dense transforms beside the folded ones)
   out->launches_per_apply = 9 + 5 * p->nchunks + ((p->interp_tile == 1 && p->ipart) ? 1 : 0) +
                             p->nchunks * ((p->cheb_tc && !(p->cheb_columns & 1) ? 1 : 0) +
                                           (p->cheb_tc_bwd ? 2 * p->cheb_tc_bwd_parts - 1 : 0));
+  for (int d = 0; d < 2; ++d)
+    if (p->cheb_fold && p->fold_thin[d] > 0 && p->fold_thin[d] < p->g.nz) out->launches_per_apply += p->nchunks;
   out->nchunks = p->nchunks;
   out->fft_col_width = 1 << p->col_lcw;
   out->fft_register_rows = p->fft_reg[0];
