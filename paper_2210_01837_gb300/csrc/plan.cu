@@ -343,33 +343,6 @@ dps_status allocate(Plan* p) {
     p->cheb_tc = p->cheb_tc && (v & 1);
     p->cheb_tc_bwd = p->cheb_tc_bwd && (v & 2);
   }
-  if (cheb_fold_applies(*p)) {
-    const dps_status fs = cheb_fold_prepare(*p);
-    if (fs == DPS_ERR_CUDA) return fs;
-    p->cheb_fold = fs == DPS_OK ? 1 : 0;
-  }
-  // factorisation table of the FP64 solve (per (kx, |ky|), filled on the legacy stream): without
-  // the memory for it the solve factorises as it goes; DPS_SOLVE_TABLE=0 chooses that by hand
-  {
-    const char* e = getenv("DPS_SOLVE_TABLE");
-    if (!(e && atoi(e) == 0)) {
-      const dps_status ft = bvp_factor_table(*p);
-      if (ft == DPS_ERR_CUDA) return ft;
-    }
-  }
-  // the tiled solve keeps its sweeps in shared memory; the thread-per-wavenumber solves need a workspace
-  p->solve_tile = p->kt.fac && solve_tile_applies(g, p->precision) ? 1 : 0;
-  if (p->solve_tile) {
-    p->bvp_blocks = solve_tile_prepare<T>(*p);
-    if (p->bvp_blocks < 1) return DPS_ERR_CUDA;
-  } else {
-    p->bvp_blocks = bvp_occupancy_blocks<T>(*p);
-    const int64_t need_blocks = (K + kBvpThreads - 1) / kBvpThreads;
-    if (p->bvp_blocks > need_blocks) p->bvp_blocks = (int)std::max<int64_t>(1, need_blocks);
-    p->ws_bytes = (int64_t)p->bvp_blocks * kBvpThreads * (int64_t)bvp_slot_bytes<T>(*p);
-    if (!alloc(&p->ws, (size_t)p->ws_bytes)) return DPS_ERR_OOM;
-  }
-  p->bvp_blocks_max = p->bvp_blocks;
   // the tile-gather interpolation's partial sums (where it applies; a variant the autotuner tries)
   if (const size_t iv = interp_tile_values(g, p->max_n)) {
     if (!alloc(&p->ipart, iv * sizeof(T))) return DPS_ERR_OOM;
@@ -406,6 +379,34 @@ dps_status allocate(Plan* p) {
     if (cudaEventCreateWithFlags(&p->ev_f[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
     if (cudaEventCreateWithFlags(&p->ev_s[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
     if (cudaEventCreateWithFlags(&p->ev_b[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
+  }
+  // Last, what a plan can run without, in the order of its worth, so that scarce memory goes to what it needs:
+  // the solve's table (per (kx, |ky|), filled on the legacy stream; without it the solve factorises as it goes;
+  // DPS_SOLVE_TABLE=0 chooses that by hand) and the folded transforms' tables (without them: dense).  The
+  // tiled solve needs its table and no workspace; the thread-per-wavenumber solves need their workspace.
+  auto workspace = [&]() -> bool {
+    p->bvp_blocks = bvp_occupancy_blocks<T>(*p);
+    const int64_t need_blocks = (K + kBvpThreads - 1) / kBvpThreads;
+    if (p->bvp_blocks > need_blocks) p->bvp_blocks = (int)std::max<int64_t>(1, need_blocks);
+    p->ws_bytes = (int64_t)p->bvp_blocks * kBvpThreads * (int64_t)bvp_slot_bytes<T>(*p);
+    return alloc(&p->ws, (size_t)p->ws_bytes);
+  };
+  const char* table = getenv("DPS_SOLVE_TABLE");
+  const bool with_table = !(table && atoi(table) == 0), tiled = with_table && solve_tile_applies(g, p->precision);
+  if (!tiled && !workspace()) return DPS_ERR_OOM;
+  if (with_table && bvp_factor_table(*p) == DPS_ERR_CUDA) return DPS_ERR_CUDA;
+  p->solve_tile = tiled && p->kt.fac ? 1 : 0;
+  if (p->solve_tile) {
+    p->bvp_blocks = solve_tile_prepare<T>(*p);
+    if (p->bvp_blocks < 1) return DPS_ERR_CUDA;
+  } else if (tiled && !workspace()) {
+    return DPS_ERR_OOM;
+  }
+  p->bvp_blocks_max = p->bvp_blocks;
+  if (cheb_fold_applies(*p)) {
+    const dps_status fs = cheb_fold_prepare(*p);
+    if (fs == DPS_ERR_CUDA) return fs;
+    p->cheb_fold = fs == DPS_OK ? 1 : 0;
   }
   return DPS_OK;
 }
