@@ -225,8 +225,9 @@ dps_status dpstokes_plan_autotune(dps_plan_t plan, int64_t n, const double* posi
 dps_status dpstokes_plan_set_fft(dps_plan_t plan, int32_t row_register, int32_t col_register, int32_t col_width);
 
 /* Sets the wavenumber-space pipeline shape by hand (no counterpart in the paper): `solve_blocks`
- * persistent blocks of the FP64 solve (1 .. the number the plan was made for, which
- * dpstokes_plan_info reports as solve_blocks right after creation) and `nchunks` column chunks
+ * persistent blocks of the FP64 solve (1 .. the number that dpstokes_plan_info reports as
+ * solve_blocks right after creation; where the tiled solve runs, also up to the grid of a thread
+ * per wavenumber, 3 blocks of 128 an SM or ceil(nkx ny / 128)) and `nchunks` column chunks
  * (1, 2, 4 or 8, at least 64 x-wavenumbers each) whose FP64 solves run on a plan-owned stream
  * beside the float transforms of the neighbouring chunks.  Results do not depend on the shape
  * beyond summation order.  DPS_ERR_INVALID_ARG (plan unchanged) when plan is NULL or a value is

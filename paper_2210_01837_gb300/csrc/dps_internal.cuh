@@ -158,7 +158,8 @@ struct Plan {
   alignas(64) unsigned char interp_tmap[128];  // CUtensorMap of the grid for the staged interpolation
   int interp_tma;       // interp_tmap holds a valid map
   int col_tma_rows;     // rows per TMA box of that pass
-  int bvp_blocks_max;   // most persistent solve blocks: what the GPU holds at once (and the workspace was allocated for)
+  int bvp_blocks_max;   // most persistent solve blocks that may be set: the larger of the chosen grid and the one of the
+                        // thread-per-wavenumber solve (the workspace's, where that solve runs)
   int solve_tile;       // the tiled solve (solve.cu) runs: a factorisation table and nz <= 128
   int interp_tile;      // interpolation variant: 0 warp per particle, 1 tile gather, 2 staged grid (where they apply)
   int cheb_tc;          // forward Chebyshev transform on the tensor cores (tcgen05, mixed precision)

@@ -384,10 +384,10 @@ dps_status allocate(Plan* p) {
   // the solve's table (per (kx, |ky|), filled on the legacy stream; without it the solve factorises as it goes;
   // DPS_SOLVE_TABLE=0 chooses that by hand) and the folded transforms' tables (without them: dense).  The
   // tiled solve needs its table and no workspace; the thread-per-wavenumber solves need their workspace.
+  const int64_t need_blocks = std::max<int64_t>(1, (K + kBvpThreads - 1) / kBvpThreads);
+  const int thread_blocks = (int)std::min<int64_t>(bvp_occupancy_blocks<T>(*p), need_blocks);
   auto workspace = [&]() -> bool {
-    p->bvp_blocks = bvp_occupancy_blocks<T>(*p);
-    const int64_t need_blocks = (K + kBvpThreads - 1) / kBvpThreads;
-    if (p->bvp_blocks > need_blocks) p->bvp_blocks = (int)std::max<int64_t>(1, need_blocks);
+    p->bvp_blocks = thread_blocks;
     p->ws_bytes = (int64_t)p->bvp_blocks * kBvpThreads * (int64_t)bvp_slot_bytes<T>(*p);
     return alloc(&p->ws, (size_t)p->ws_bytes);
   };
@@ -402,7 +402,7 @@ dps_status allocate(Plan* p) {
   } else if (tiled && !workspace()) {
     return DPS_ERR_OOM;
   }
-  p->bvp_blocks_max = p->bvp_blocks;
+  p->bvp_blocks_max = std::max(p->bvp_blocks, thread_blocks);  // any grid is right for the tiled solve
   if (cheb_fold_applies(*p)) {
     const dps_status fs = cheb_fold_prepare(*p);
     if (fs == DPS_ERR_CUDA) return fs;

@@ -110,3 +110,27 @@ def test_either_side_of_the_rule_matches_the_general_solve(mode, precision, nx, 
     U_ref, _ = gpu_mobility(params, pos, F, None, precision, plan=general)
     general.close()
     assert rel_l2(U, U_ref) <= TOL[precision]
+
+
+@pytest.mark.parametrize("nx,ny,nz,precision", [(384, 384, 65, "mixed"), (40, 36, 33, "fp64"), (16, 12, 8, "mixed")])
+def test_every_grid_of_the_thread_per_wavenumber_solve_is_accepted(nx, ny, nz, precision, monkeypatch):
+    """Grids set for that solve (three blocks an SM, or all wavenumbers' blocks) hold for the tiled one too,
+    which may choose fewer; blocks without a tile leave the result as it is."""
+    params = small_params("slit", nx=nx, ny=ny, nz=nz, zmax=6.0, torque=False)
+    pos, F, _ = random_particles(params, 9, seed=nz, torques=False)
+    kw = dict(with_torque=False, precision=precision, max_n=len(pos))
+    monkeypatch.setenv("DPS_SOLVE_TABLE", "0")
+    general = binding.Plan.from_params(params, **kw)
+    most = general.info().solve_blocks
+    general.close()
+    monkeypatch.delenv("DPS_SOLVE_TABLE")
+    plan = binding.Plan.from_params(params, **kw)
+    own = plan.info().solve_blocks
+    U0, _ = gpu_mobility(params, pos, F, None, precision, plan=plan)
+    for blocks in {most, max(1, most // 2), own}:
+        plan.set_pipeline(blocks, 1)
+        U, _ = gpu_mobility(params, pos, F, None, precision, plan=plan)
+        assert (U == U0).all()
+    with pytest.raises(binding.DpsError):
+        plan.set_pipeline(max(most, own) + 1, 1)
+    plan.close()
