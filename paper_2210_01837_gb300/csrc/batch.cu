@@ -165,7 +165,7 @@ struct Server {
 
   // plan sizing before creation, following the plan's own allocations: grid, particle records and
   // bins, solve workspace, spectra, staging buffers and tables (an upper bound, plus 1/8)
-  static int64_t estimate_bytes(const dps_serve_request& r) {
+  static int64_t estimate_bytes(const dps_serve_request& r, bool lean) {
     const int64_t ts = r.kp.precision == DPS_MIXED ? 4 : 8;
     const int64_t nx = r.grid.nx, ny = r.grid.ny, nz = r.grid.nz;
     const int64_t nkx = nx / 2 + 1, pitch = (nkx + 31) / 32 * 32, K = nkx * ny;
@@ -184,12 +184,12 @@ struct Server {
     for (double x : {r.walls.slip_bottom, r.walls.slip_top, r.walls.uw_bottom[0], r.walls.uw_bottom[1],
                      r.walls.uw_top[0], r.walls.uw_top[1]})
       g.slip = g.slip || x != 0.0;
-    if (solve_tile_applies(g, r.kp.precision))  // the tiled solve's table; else workspace and factorisation table
-      b += (int64_t)solve_tile_table_bytes(g, r.kp.precision);
-    else
-      b += blocks * kBvpThreads * nz * (3 * 16 + 3 * 8 + 2 * ts) + nkx * (ny / 2 + 1) * nz * 4 * 8;
+    // the tiled solve's table, or the other's workspace and factorisation table (a lean plan takes the smaller)
+    const int64_t thread = blocks * kBvpThreads * nz * (3 * 16 + 3 * 8 + 2 * ts) + nkx * (ny / 2 + 1) * nz * 4 * 8;
+    const int64_t tile = solve_tile_applies(g, r.kp.precision) ? (int64_t)solve_tile_table_bytes(g, r.kp.precision) : -1;
+    b += tile >= 0 && (!lean || tile < thread) ? tile : thread;
     b += 3 * nz * K * 2 * ts + 12 * K * 2 * ts;                          // kbuf, kaux
-    if (ts == 8) b += nkx * (ny / 2 + 1) * nz * 16 + 256 * nz * nz;      // the folded transforms' tables
+    if (!lean && cheb_fold_applies(g, r.kp.precision)) b += (int64_t)cheb_fold_bytes(g);
     // partial sums of the tile-gather interpolation (forces only, or equal supports with the
     // spectral curl): slots of the tiles a support can overlap x fields x particles
     const int64_t ifields = route == DPS_TORQUE_NONE ? 3
@@ -355,7 +355,9 @@ struct Server {
             if (!find_any(key_of(queue[i].r))) { pick = i; break; }
           if (pick == window) break;  // every candidate's plan is busy: wait for a completion
           Pending q = queue[pick];
-          const int64_t need = estimate_bytes(q.r);
+          int64_t need = estimate_bytes(q.r, false);
+          const bool lean = need > budget;  // then as small as a plan gets
+          if (lean) need = estimate_bytes(q.r, true);
           if (need > budget) {  // can never fit
             queue.erase(queue.begin() + pick);
             fail(q, DPS_ERR_OOM);
@@ -370,8 +372,8 @@ struct Server {
             continue;
           }
           dps_plan_t plan = nullptr;
-          const dps_status st = dpstokes_plan_create_ex(&plan, q.r.Lx, q.r.Ly, q.r.zmin, q.r.zmax, q.r.wall_mode,
-                                                        &q.r.grid, &q.r.kp, &q.r.walls);
+          const dps_status st = plan_create(&plan, q.r.Lx, q.r.Ly, q.r.zmin, q.r.zmax, q.r.wall_mode, &q.r.grid,
+                                            &q.r.kp, &q.r.walls, lean);
           if (st != DPS_OK) {
             queue.erase(queue.begin() + pick);
             fail(q, st);

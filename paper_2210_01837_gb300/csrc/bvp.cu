@@ -1660,7 +1660,6 @@ void launch_bvp(const Plan& p, int part, int kx0, int w, cudaStream_t s) {
 
 dps_status bvp_factor_table(Plan& p) {
   const Geometry& g = p.g;
-  if (solve_tile_applies(g, p.precision)) return solve_tile_table(p);
   const int64_t KP = (int64_t)g.nkx * (g.ny / 2 + 1);
   const size_t bytes = (size_t)KP * g.nz * 4 * sizeof(double);
   void* q = nullptr;

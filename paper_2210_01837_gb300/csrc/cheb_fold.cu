@@ -465,9 +465,8 @@ auto fold_dispatch(int bucket, F&& f) {
 
 }  // namespace
 
-bool cheb_fold_applies(const Plan& p) {
-  const Geometry& g = p.g;
-  return p.precision == DPS_FP64 && (g.nz - 1) % 8 == 0 && g.nz >= 9 && g.nz <= 129;
+bool cheb_fold_applies(const Geometry& g, int precision) {
+  return precision == DPS_FP64 && (g.nz - 1) % 8 == 0 && g.nz >= 9 && g.nz <= 129;
 }
 
 // Folding transforms whole columns; the dense kernels only read (forward) or form (backward) the occupied

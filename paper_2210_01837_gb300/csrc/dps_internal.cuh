@@ -160,6 +160,7 @@ struct Plan {
   int col_tma_rows;     // rows per TMA box of that pass
   int bvp_blocks_max;   // most persistent solve blocks that may be set: the larger of the chosen grid and the one of the
                         // thread-per-wavenumber solve (the workspace's, where that solve runs)
+  int lean;             // the serving loop's budget is short: no folded transforms, and the smaller of the solves' forms
   int solve_tile;       // the tiled solve (solve.cu) runs: a factorisation table and nz <= 128
   int interp_tile;      // interpolation variant: 0 warp per particle, 1 tile gather, 2 staged grid (where they apply)
   int cheb_tc;          // forward Chebyshev transform on the tensor cores (tcgen05, mixed precision)
@@ -268,6 +269,10 @@ double es_norm(double alpha, double beta);
 double es_deriv_cut(double alpha, double beta);
 dps_status particle_geometry(Geometry& g, const dps_kernel_params* kp, int tsize);
 
+// dpstokes_plan_create_ex, as small as a plan gets with lean
+dps_status plan_create(dps_plan_t* out, double Lx, double Ly, double zmin, double zmax, int32_t wall_mode,
+                       const dps_grid* grid, const dps_kernel_params* kp, const dps_wall_params* wp, bool lean);
+
 // launchers (stream-ordered, no host sync)
 template <typename T> void launch_records(const Plan& p, int64_t n, const double* pos, const double* F,
                                           const double* Tq, cudaStream_t s);
@@ -313,7 +318,7 @@ int cheb_columns_applies(const Plan& p);
 void launch_cheb_columns(const Plan& p, bool backward, int kx0, int w, cudaStream_t s);
 // the folded transforms (cheb_fold.cu): where they apply, the bytes of their tables, their preparation (DPS_ERR_OOM
 // leaves the plan on the lane kernels) and launcher
-bool cheb_fold_applies(const Plan& p);
+bool cheb_fold_applies(const Geometry& g, int precision);
 size_t cheb_fold_bytes(const Geometry& g);
 dps_status cheb_fold_prepare(Plan& p);
 void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t s);

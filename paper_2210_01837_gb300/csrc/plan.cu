@@ -392,9 +392,14 @@ dps_status allocate(Plan* p) {
     return alloc(&p->ws, (size_t)p->ws_bytes);
   };
   const char* table = getenv("DPS_SOLVE_TABLE");
-  const bool with_table = !(table && atoi(table) == 0), tiled = with_table && solve_tile_applies(g, p->precision);
+  const bool with_table = !(table && atoi(table) == 0);
+  bool tiled = with_table && solve_tile_applies(g, p->precision);
+  if (p->lean)
+    tiled = tiled && solve_tile_table_bytes(g, p->precision) <=
+                         (size_t)thread_blocks * kBvpThreads * bvp_slot_bytes<T>(*p) +
+                             (size_t)g.nkx * (g.ny / 2 + 1) * g.nz * 4 * sizeof(double);
   if (!tiled && !workspace()) return DPS_ERR_OOM;
-  if (with_table && bvp_factor_table(*p) == DPS_ERR_CUDA) return DPS_ERR_CUDA;
+  if (with_table && (tiled ? solve_tile_table(*p) : bvp_factor_table(*p)) == DPS_ERR_CUDA) return DPS_ERR_CUDA;
   p->solve_tile = tiled && p->kt.fac ? 1 : 0;
   if (p->solve_tile) {
     p->bvp_blocks = solve_tile_prepare<T>(*p);
@@ -403,7 +408,7 @@ dps_status allocate(Plan* p) {
     return DPS_ERR_OOM;
   }
   p->bvp_blocks_max = std::max(p->bvp_blocks, thread_blocks);  // any grid is right for the tiled solve
-  if (cheb_fold_applies(*p)) {
+  if (!p->lean && cheb_fold_applies(g, p->precision)) {
     const dps_status fs = cheb_fold_prepare(*p);
     if (fs == DPS_ERR_CUDA) return fs;
     p->cheb_fold = fs == DPS_OK ? 1 : 0;
@@ -528,11 +533,18 @@ const char* dpstokes_error_string(dps_status st) {
 
 dps_status dpstokes_plan_create(dps_plan_t* out, double Lx, double Ly, double zmin, double zmax, int32_t wall_mode,
                                 const dps_grid* grid, const dps_kernel_params* kp) {
-  return dpstokes_plan_create_ex(out, Lx, Ly, zmin, zmax, wall_mode, grid, kp, nullptr);
+  return dps::plan_create(out, Lx, Ly, zmin, zmax, wall_mode, grid, kp, nullptr, false);
 }
 
 dps_status dpstokes_plan_create_ex(dps_plan_t* out, double Lx, double Ly, double zmin, double zmax, int32_t wall_mode,
                                    const dps_grid* grid, const dps_kernel_params* kp, const dps_wall_params* wp) {
+  return dps::plan_create(out, Lx, Ly, zmin, zmax, wall_mode, grid, kp, wp, false);
+}
+
+}  // extern "C"
+
+dps_status dps::plan_create(dps_plan_t* out, double Lx, double Ly, double zmin, double zmax, int32_t wall_mode,
+                            const dps_grid* grid, const dps_kernel_params* kp, const dps_wall_params* wp, bool lean) {
   if (!out) return DPS_ERR_INVALID_ARG;
   *out = nullptr;
   if (!grid || !kp) return DPS_ERR_INVALID_ARG;
@@ -580,6 +592,7 @@ dps_status dpstokes_plan_create_ex(dps_plan_t* out, double Lx, double Ly, double
   cudaGetDevice(&p->device);
   p->precision = kp->precision;
   p->max_n = kp->max_n;
+  p->lean = lean;
   p->g = g;
   if (!dps::fft_plan(nx, p->fx) || !dps::fft_plan(ny, p->fy) || !dps::fft_plan_balanced(nx, p->fxr) ||
       !dps::fft_plan_balanced(ny, p->fyr)) {
@@ -597,6 +610,8 @@ dps_status dpstokes_plan_create_ex(dps_plan_t* out, double Lx, double Ly, double
   *out = reinterpret_cast<dps_plan_t>(p);
   return DPS_OK;
 }
+
+extern "C" {
 
 dps_status dpstokes_apply(dps_plan_t plan, int64_t n, const double* positions, const double* forces,
                           const double* torques, double* out_vel, double* out_angvel, void* stream) {

@@ -238,3 +238,32 @@ def test_server_queue_limit_refuses_and_still_serves():
     assert refused >= 1 and stats["rejected"] == refused
     assert len(accepted) + refused == 12
     srv.close()
+
+
+@pytest.mark.parametrize("mode,nx,ny,nz,precision", [("slit", 384, 384, 97, "fp64"), ("free", 400, 384, 65, "fp64"),
+                                                    ("slit", 64, 48, 33, "mixed")])
+def test_server_serves_within_the_budget_of_a_plan_without_extra_tables(mode, nx, ny, nz, precision):
+    """The folded transforms and the tiled solve keep tables that a plan can run without: a budget that holds
+    the grid, spectra, workspace and factorisation table (its size as the server reckons it, with an eighth
+    for rounding) serves the request, and the plan stays within it."""
+    n, ts = 20, 8 if precision == "fp64" else 4
+    params = small_params(mode, nx=nx, ny=ny, nz=nz, zmax=8.0, torque=False)
+    pos, F, _ = random_particles(params, n, seed=nz, torques=False)
+    U_ref, _ = _alone(params, pos, F, None, precision, False)
+    nkx, pitch, K = nx // 2 + 1, (nx // 2 + 32) // 32 * 32, (nx // 2 + 1) * ny
+    bx, by = -(-nx // 32), -(-ny // 8)
+    b = 3 * nz * ny * pitch * 2 * ts
+    b += n * (4 * (8 + (6 + 26 + nz) * ts // 4 + 3) + 8 + 15 * 8) + 3 * bx * by * 4
+    b += min(608, -(-K // 128)) * 128 * nz * (3 * 16 + 3 * 8 + 2 * ts)
+    b += 3 * nz * K * 2 * ts + 12 * K * 2 * ts + nkx * (ny // 2 + 1) * nz * 4 * 8
+    b += min(bx, 2 + (nx % 32 != 0)) * min(by, 2 + (ny % 8 != 0)) * 3 * n * ts
+    b += 8 * nz * (nz + 32) * ts + 3 * (nx + ny) * 16 + 16 * nz * 8
+    budget = b + b // 8 + (256 << 10)
+    srv = binding.Server(memory_budget_bytes=budget, slots=1)
+    t = srv.submit(params, with_torque=False, precision=precision, max_n=n, pos=_pinned(pos), F=_pinned(F))
+    r, U, _ = srv.wait(t, timeout_s=60.0)
+    resident = srv.stats()["bytes_resident"]
+    srv.close()
+    assert r.status == binding.DPS_OK
+    assert resident <= budget
+    assert rel_l2(U, U_ref) <= {"fp64": 1e-9, "mixed": 1e-5}[precision]
