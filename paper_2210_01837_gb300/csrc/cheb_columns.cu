@@ -11,6 +11,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "bvp_device.cuh"
 #include "dps_internal.cuh"
@@ -188,24 +189,34 @@ __global__ void __launch_bounds__(kColThreads, col_blocks(HP)) cols_bwd_kernel(c
   }
 }
 
-template <typename KernelT>
-unsigned cols_grid(const Plan& p, KernelT kernel, size_t smem, int w) {
-  int per_sm = 0, sms = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kColThreads, smem);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device);
+// blocks of a launch: of the chunk's columns, no more than the GPU holds at once
+unsigned cols_blocks(const Plan& p, bool backward, int w) {
   const int64_t blocks = 3 * (((int64_t)w * p.g.ny + kColThreads - 1) / kColThreads);
-  return (unsigned)std::min<int64_t>(blocks, (int64_t)std::max(1, per_sm) * std::max(1, sms));
+  return (unsigned)std::min<int64_t>(blocks, p.cols_grid[backward]);
+}
+template <int HP>
+size_t cols_smem(const Geometry& g, bool backward) {
+  return ((size_t)(g.nz + 1) / 2 * 2 * HP + (backward ? g.nz : 0)) * sizeof(float);
 }
 
 template <int HP, int CORR>
 void launch_bwd(const Plan& p, int kx0, int w, cudaStream_t s) {
   const Geometry& g = p.g;
-  const size_t smem = ((size_t)(g.nz + 1) / 2 * 2 * HP + g.nz) * sizeof(float);
-  cols_bwd_kernel<HP, CORR><<<cols_grid(p, cols_bwd_kernel<HP, CORR>, smem, w), kColThreads, smem, s>>>(
+  cols_bwd_kernel<HP, CORR><<<cols_blocks(p, true, w), kColThreads, cols_smem<HP>(g, true), s>>>(
       g, reinterpret_cast<const float*>(p.kt.ict), p.kt.cpad, reinterpret_cast<const float*>(p.tab.zeta),
       reinterpret_cast<const cplx<float>*>(p.kt.kbuf), reinterpret_cast<const cplx<float>*>(p.kt.kaux),
       reinterpret_cast<cplx<float>*>(p.grid), p.zrange, kx0, w, M_PI / g.Lx, M_PI / g.Ly,
       (float)(1.0 / ((double)g.nx * (double)g.ny)));
+}
+
+// f(std::integral_constant<int, HP>) for the column's bucket
+template <typename F>
+auto with_bucket(const Geometry& g, F&& f) {
+  const int half = (g.nz + 1) / 2;
+  if (half <= 10) return f(std::integral_constant<int, 10>());
+  if (half <= 18) return f(std::integral_constant<int, 18>());
+  if (half <= 26) return f(std::integral_constant<int, 26>());
+  return f(std::integral_constant<int, 34>());  // (backward only)
 }
 
 template <int HP>
@@ -213,8 +224,7 @@ void launch_dir(const Plan& p, bool backward, int kx0, int w, cudaStream_t s) {
   const Geometry& g = p.g;
   if constexpr (HP <= 26) {
     if (!backward) {
-      const size_t smem = (size_t)(g.nz + 1) / 2 * 2 * HP * sizeof(float);
-      cols_fwd_kernel<HP><<<cols_grid(p, cols_fwd_kernel<HP>, smem, w), kColThreads, smem, s>>>(
+      cols_fwd_kernel<HP><<<cols_blocks(p, false, w), kColThreads, cols_smem<HP>(g, false), s>>>(
           g, reinterpret_cast<const float*>(p.kt.ct), p.kt.npad, reinterpret_cast<const cplx<float>*>(p.grid),
           reinterpret_cast<cplx<float>*>(p.kt.kbuf), p.zrange, kx0, w);
       return;
@@ -241,17 +251,33 @@ void launch_dir(const Plan& p, bool backward, int kx0, int w, cudaStream_t s) {
 // its angular velocities came out 9 % further from double (33 nodes: 4.9e-7 against 5.4e-7; linear velocities
 // 4.5e-7 against 3.8e-7).  Without torques both directions together are closer (19 nodes 3.7e-7 -> 3.5e-7, 49
 // nodes 5.4e-7 -> 4.6e-7).
-int cheb_columns_applies(const Plan& p) {
-  if (p.precision != DPS_MIXED || p.g.spectral_curl) return 0;
-  return (p.g.nz <= 52 && !p.g.with_torque ? 1 : 0) | (p.g.nz <= 68 ? 2 : 0);
+int cheb_columns_prepare(Plan& p) {
+  const Geometry& g = p.g;
+  p.cheb_columns = 0;
+  if (p.precision != DPS_MIXED || g.spectral_curl) return 1;
+  p.cheb_columns = (g.nz <= 52 && !g.with_torque ? 1 : 0) | (g.nz <= 68 ? 2 : 0);
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device) != cudaSuccess) return 0;
+  return with_bucket(g, [&](auto hp) {
+    constexpr int HP = decltype(hp)::value;
+    const void* kernel[2] = {nullptr, g.mode == DPS_FREE   ? (const void*)cols_bwd_kernel<HP, 0>
+                                      : g.mode == DPS_SLIT ? (const void*)cols_bwd_kernel<HP, 2>
+                                                           : (const void*)cols_bwd_kernel<HP, 1>};
+    if constexpr (HP <= 26) kernel[0] = (const void*)cols_fwd_kernel<HP>;
+    for (int d = 0; d < 2; ++d) {
+      int per_sm = 0;
+      if (!(p.cheb_columns >> d & 1)) continue;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel[d], kColThreads, cols_smem<HP>(g, d == 1)) !=
+              cudaSuccess || per_sm < 1)
+        return 0;
+      p.cols_grid[d] = per_sm * sms;
+    }
+    return 1;
+  });
 }
 
 void launch_cheb_columns(const Plan& p, bool backward, int kx0, int w, cudaStream_t s) {
-  const int half = (p.g.nz + 1) / 2;
-  if (half <= 10) launch_dir<10>(p, backward, kx0, w, s);
-  else if (half <= 18) launch_dir<18>(p, backward, kx0, w, s);
-  else if (half <= 26) launch_dir<26>(p, backward, kx0, w, s);
-  else launch_dir<34>(p, backward, kx0, w, s);  // (backward only)
+  with_bucket(p.g, [&](auto hp) { launch_dir<decltype(hp)::value>(p, backward, kx0, w, s); });
 }
 
 }  // namespace dps

@@ -504,6 +504,10 @@ dps_status cheb_fold_prepare(Plan& p) {
     return g.spectral_curl ? fold_allow<T, true, HP>() : fold_allow<T, false, HP>();
   });
   if (!ok) return DPS_ERR_CUDA;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device) != cudaSuccess) return DPS_ERR_CUDA;
+  const int nf = g.spectral_curl ? 5 : 3;
+  p.fold_grid = sms * (2 * (fold_smem<T>(g.nz, nf) + 1024) <= 228 * 1024 && nf == 3 ? 2 : 1);
   const size_t nt = fold_table_values<T>(g.nz), bytes = cheb_fold_bytes(g);
   void* q = nullptr;
   if (cudaMalloc(&q, bytes) != cudaSuccess) {
@@ -529,8 +533,6 @@ dps_status cheb_fold_prepare(Plan& p) {
 void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t s) {
   using T = double;
   const Geometry& g = p.g;
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device);
   const int64_t tiles = ((int64_t)w * g.ny + kFoldK - 1) / kFoldK;
   const size_t nt = fold_table_values<T>(g.nz);
   cplx<T>* grid = reinterpret_cast<cplx<T>*>(p.grid);
@@ -538,8 +540,7 @@ void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t
   const cplx<T>* kaux = reinterpret_cast<const cplx<T>*>(p.kt.kaux);
   const int nf = g.spectral_curl ? 5 : 3;
   const size_t smem = fold_smem<T>(g.nz, nf);
-  const int per_sm = 2 * (smem + 1024) <= 228 * 1024 && nf == 3 ? 2 : 1;
-  const unsigned blocks = (unsigned)(tiles < (int64_t)sms * per_sm ? tiles : (int64_t)sms * per_sm);
+  const unsigned blocks = (unsigned)(tiles < p.fold_grid ? tiles : p.fold_grid);
   const double2* ecf = g.mode != DPS_FREE ? reinterpret_cast<const double2*>(p.kt.fold + 2 * nt) : nullptr;
   const int64_t KP = (int64_t)g.nkx * (g.ny / 2 + 1);
   const double hx = M_PI / g.Lx, hy = M_PI / g.Ly;

@@ -165,8 +165,10 @@ struct Plan {
   int interp_tile;      // interpolation variant: 0 warp per particle, 1 tile gather, 2 staged grid (where they apply)
   int cheb_tc;          // forward Chebyshev transform on the tensor cores (tcgen05, mixed precision)
   int cheb_columns;     // three-field float transforms in registers: bit 0 forward, bit 1 backward
+  int cols_grid[2];     // their resident grids
   int cheb_tc_bwd;      // backward Chebyshev transform on the tensor cores (spectral-curl torques)
   int cheb_fold;        // Chebyshev transforms by folding (double precision, nz - 1 a multiple of 8)
+  int fold_grid;        // their resident grid
   int fold_thin[2];     // forward, backward: most occupied planes at which the dense transforms run instead
   int cheb_tc_bwd_parts;  // launches of the backward transform (output planes split beyond 96 nodes)
   int cheb_tc_grid;     // persistent blocks of that kernel
@@ -312,9 +314,9 @@ int cheb_tc_prepare(Plan& p);
 void launch_cheb_fwd_tc(const Plan& p, int kx0, int w, cudaStream_t s);
 void launch_cheb_bwd_tc(const Plan& p, int kx0, int w, cudaStream_t s);
 int cheb_tc_np(const Geometry& g);
-// the transforms of three float fields in registers (cheb_columns.cu): where they apply (bit 0 forward, bit 1
-// backward)
-int cheb_columns_applies(const Plan& p);
+// the transforms of three float fields in registers (cheb_columns.cu): readiness (sets cheb_columns where they
+// apply, and their grids; 0 on a CUDA error) and launcher
+int cheb_columns_prepare(Plan& p);
 void launch_cheb_columns(const Plan& p, bool backward, int kx0, int w, cudaStream_t s);
 // the folded transforms (cheb_fold.cu): where they apply, the bytes of their tables, their preparation (DPS_ERR_OOM
 // leaves the plan on the lane kernels) and launcher

@@ -336,7 +336,7 @@ dps_status allocate(Plan* p) {
   if (!cheb_tc_prepare(*p)) return DPS_ERR_CUDA;
   if (p->cheb_tc && !alloc((void**)&p->kt.bimg_f, cheb_tc_image_bytes(g, false))) return DPS_ERR_OOM;
   if (p->cheb_tc_bwd && !alloc((void**)&p->kt.bimg_b, cheb_tc_image_bytes(g, true))) return DPS_ERR_OOM;
-  p->cheb_columns = cheb_columns_applies(*p);
+  if (!cheb_columns_prepare(*p)) return DPS_ERR_CUDA;
   if (const char* e = getenv("DPS_CHEB_TC")) {  // bit 0 forward, bit 1 backward
     const int v = atoi(e);
     p->cheb_columns &= 2;
