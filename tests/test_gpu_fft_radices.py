@@ -35,3 +35,29 @@ def test_every_radix_in_every_variant_matches_oracle(nx, ny):
                     assert rel_l2(W, W_ref) <= TOL[precision], (precision, rows, cols, width)
         assert tried >= 8
         plan.close()
+
+
+@pytest.mark.parametrize("nx", [
+    3136, 3584,  # last stage 14 (float rows' default there), first 16
+    1600, 2240,  # last stage 10
+    384,         # last stage 6
+    896, 1344,   # first stage 14
+    640,         # first stage 10
+])
+def test_paired_first_and_last_stages_match_oracle(nx):
+    """Register-staged rows whose last stage splits the half spectra and whose first stage joins them in
+    registers: spans that are multiples of 32, at the composite radices; an odd row count leaves one row
+    without a partner."""
+    params = small_params("bottom_wall", nx=nx, ny=15, nz=9, zmax=4.0, torque=True)
+    pos, F, T = random_particles(params, 12, seed=nx)
+    U_ref, W_ref = mobility(oracle_params(params), pos, F, T)
+    for precision in ("fp64", "mixed"):
+        plan = binding.Plan.from_params(params, with_torque=True, precision=precision, max_n=len(pos))
+        info = plan.info()
+        if precision == "mixed" and nx >= 3136:
+            assert info.fft_register_rows == 1
+        plan.set_fft(1, info.fft_register_cols, info.fft_col_width)
+        U, W = gpu_mobility(params, pos, F, T, precision, plan=plan)
+        plan.close()
+        assert rel_l2(U, U_ref) <= TOL[precision], precision
+        assert rel_l2(W, W_ref) <= TOL[precision], precision
