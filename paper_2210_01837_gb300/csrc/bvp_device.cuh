@@ -1,4 +1,4 @@
-// Device helpers shared by the per-wavenumber kernels (bvp.cu) and the tiled solve (solve.cu):
+// Device helpers shared by the per-wavenumber kernels (bvp.cu, solve.cu, cheb_fold.cu, cheb_columns.cu):
 // conversions on the integer pipe, streaming accesses, the wavenumber of a spectrum column and the
 // wall-correction amplitudes.
 #pragma once
@@ -56,6 +56,7 @@ __device__ __forceinline__ void st_stream(cplx<float>* p, cplx<float> v) {
 __device__ __forceinline__ void st_stream(cplx<double>* p, cplx<double> v) {
   __stcs(reinterpret_cast<double2*>(p), make_double2(v.x, v.y));
 }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 template <typename T> __device__ __forceinline__ cplx<double> wid(cplx<T> a) { return mk<double>(widen<T>(a.x), widen<T>(a.y)); }
 template <typename T> __device__ __forceinline__ cplx<T> nar(cplx<double> a) { return mk<T>(narrow<T>(a.x), narrow<T>(a.y)); }

@@ -32,11 +32,10 @@
 namespace dps {
 namespace {
 
+using T = double;           // the plans that fold
 constexpr int kFoldK = 16;  // wavenumbers per block
 
-template <typename T> __host__ __device__ constexpr int fold_pad(int hp) {  // table row: whole 16-byte loads
-  return sizeof(T) == 8 ? (hp + 1) / 2 * 2 : (hp + 3) / 4 * 4;
-}
+__host__ __device__ constexpr int fold_pad(int hp) { return (hp + 1) / 2 * 2; }  // table row: whole 16-byte loads
 // outputs of a part kept in registers: h/2 + 1, by buckets
 __host__ __device__ inline int fold_bucket(int N) { return N <= 33 ? 5 : (N <= 65 ? 9 : (N <= 97 ? 13 : 17)); }
 
@@ -60,16 +59,15 @@ __host__ __device__ inline FoldPart fold_part_of(int r, int q, int h) {
   }
 }
 __host__ __device__ inline int fold_rows(int h) { return 2 * h + 6 * (h / 2) + 1; }
-template <typename T> __host__ __device__ inline size_t fold_table_values(int N) {
-  return (size_t)fold_rows((N - 1) / 4) * fold_pad<T>(fold_bucket(N));
+__host__ __device__ inline size_t fold_table_values(int N) {
+  return (size_t)fold_rows((N - 1) / 4) * fold_pad(fold_bucket(N));
 }
 // shared memory: fields, part tables, derivative factors
-template <typename T> __host__ __device__ inline size_t fold_smem(int N, int nf) {
-  return ((size_t)nf * N * 32 + fold_table_values<T>(N) + N) * sizeof(T);
+__host__ __device__ inline size_t fold_smem(int N, int nf) {
+  return ((size_t)nf * N * 32 + fold_table_values(N) + N) * sizeof(T);
 }
 
 // x_c -> p_c, q_c, o_c, o_{M-c} of one column in place, c = 0 .. h: slots c, M - c, n1 - c, M + c; returns p_c
-template <typename T>
 __device__ __forceinline__ T fold_quad(T* x, int c, int h) {
   const int M = 2 * h, n1 = 4 * h;
   const T a = x[c * 32], b = x[(n1 - c) * 32];
@@ -86,7 +84,6 @@ __device__ __forceinline__ T fold_quad(T* x, int c, int h) {
   return e + f;
 }
 // work item c = 0 .. h/2: the quadruples of c and h - c, then s_c in slot c and d_c in slot h - c
-template <typename T>
 __device__ __forceinline__ void fold_in(T* x, int c, int h) {
   const T a = fold_quad(x, c, h);
   if (2 * c == h) {
@@ -99,7 +96,6 @@ __device__ __forceinline__ void fold_in(T* x, int c, int h) {
 }
 
 // X_n from the parts' outputs: X_{4j} in slot j, X_{4j+2} in slot M - j, E_m in slot n1 - 2m, O_m below it
-template <typename T>
 __device__ __forceinline__ T fold_out(const T* x, int n, int M) {
   if (!(n & 1)) return x[((n & 2) ? M - (n >> 2) : n >> 2) * 32];
   const bool up = n < M;
@@ -108,9 +104,9 @@ __device__ __forceinline__ T fold_out(const T* x, int n, int M) {
   return up ? e + o : e - o;
 }
 
-template <typename T, int HP>
+template <int HP>
 __device__ __forceinline__ void fold_dot(const T* x, const T* __restrict__ tab, const FoldPart& p, T (&acc)[HP]) {
-  constexpr int PAD = fold_pad<T>(HP), V = 16 / sizeof(T);
+  constexpr int PAD = fold_pad(HP);
 #pragma unroll
   for (int j = 0; j < HP; ++j) acc[j] = (T)0;
   const T* xi = x + p.x0 * 32;
@@ -120,29 +116,17 @@ __device__ __forceinline__ void fold_dot(const T* x, const T* __restrict__ tab, 
     const T v = *xi;
     xi += step;
 #pragma unroll
-    for (int j = 0; j < PAD; j += V) {
-      T t[V];
-      if constexpr (sizeof(T) == 8) {
-        const double2 u = *reinterpret_cast<const double2*>(row + j);
-        t[0] = u.x;
-        t[1] = u.y;
-      } else {
-        const float4 u = *reinterpret_cast<const float4*>(row + j);
-        t[0] = u.x;
-        t[1] = u.y;
-        t[2] = u.z;
-        t[3] = u.w;
-      }
-#pragma unroll
-      for (int k = 0; k < V; ++k)
-        if (j + k < HP) acc[j + k] = fma(t[k], v, acc[j + k]);
+    for (int j = 0; j < PAD; j += 2) {
+      const double2 t = *reinterpret_cast<const double2*>(row + j);
+      acc[j] = fma(t.x, v, acc[j]);
+      if (j + 1 < HP) acc[j + 1] = fma(t.y, v, acc[j + 1]);
     }
     row += PAD;
   }
 }
 
 // Folds the columns of all fields and applies their parts, in place; by the whole block, between barriers.
-template <typename T, int HP>
+template <int HP>
 __device__ __forceinline__ void fold_apply(T* sx, const T* tab, int N) {
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, f = wi >> 2, h = (N - 1) / 4, k = h / 2, M = 2 * h;
   const int r = (wi + f) & 3;  // a field's roles on all sub-partitions, a role of the fields too
@@ -150,8 +134,8 @@ __device__ __forceinline__ void fold_apply(T* sx, const T* tab, int N) {
   for (int c = wi & 3; c <= k; c += 4) fold_in(x, c, h);
   __syncthreads();
   T a[HP], b[HP];
-  fold_dot<T, HP>(x, tab, fold_part_of(r, 0, h), a);
-  fold_dot<T, HP>(x, tab, fold_part_of(r, 1, h), b);
+  fold_dot<HP>(x, tab, fold_part_of(r, 0, h), a);
+  fold_dot<HP>(x, tab, fold_part_of(r, 1, h), b);
   __syncthreads();  // inputs read
 #pragma unroll
   for (int j = 0; j < HP; ++j) {
@@ -171,8 +155,6 @@ __device__ __forceinline__ void fold_apply(T* sx, const T* tab, int N) {
   }
   __syncthreads();
 }
-
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 struct FoldLane {
   int64_t col;   // spectrum column in a plane (complex), -1 beyond the end
@@ -204,7 +186,7 @@ __device__ __forceinline__ FoldLane fold_lane(const Geometry& g, int64_t it, int
 
 // forward: kbuf[o][n][k] = (C a_o + D C b_o)[n] with a_o = f_o + (1/2)(i k x tau)_o, b_x = -tau_y / 2,
 // b_y = tau_x / 2 (TQ; else a_o = f_o alone)
-template <typename T, bool TQ, int HP>
+template <bool TQ, int HP>
 __global__ void __launch_bounds__((TQ ? 20 : 12) * 32) fold_fwd_kernel(const __grid_constant__ Geometry g,
                                                                       const T* __restrict__ tab_g,
                                                                       const cplx<T>* __restrict__ grid,
@@ -217,9 +199,9 @@ __global__ void __launch_bounds__((TQ ? 20 : 12) * 32) fold_fwd_kernel(const __g
   const int N = g.nz, M = (N - 1) / 2;
   T* sx = reinterpret_cast<T*>(smraw);  // [NF][N][32]
   T* tab = sx + (size_t)NF * N * 32;
-  T* dn = tab + fold_table_values<T>(N);  // [N] 2 (n + 1) d/dz s, times the half of the curl forward
+  T* dn = tab + fold_table_values(N);  // [N] 2 (n + 1) d/dz s, times the half of the curl forward
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, part = lane >> 4, kc = lane & 15;
-  const int nt = (int)fold_table_values<T>(N);
+  const int nt = (int)fold_table_values(N);
   for (int i = threadIdx.x; i < nt; i += NW * 32) tab[i] = tab_g[i];
   for (int i = threadIdx.x; i < N; i += NW * 32) dn[i] = (T)((i + 1 == N - 1 ? 0.25 : 0.5) * (2 * (i + 1)) * g.sH);
   const int64_t K = (int64_t)g.nkx * g.ny, total = (int64_t)w * g.ny;
@@ -265,7 +247,7 @@ __global__ void __launch_bounds__((TQ ? 20 : 12) * 32) fold_fwd_kernel(const __g
           for (int f = part; f < (TQ ? 6 : 3); f += 2) prefetch_l2(q + ((size_t)f * g.nz + c) * plane);
     }
     __syncthreads();
-    fold_apply<T, HP>(sx, tab, N);
+    fold_apply<HP>(sx, tab, N);
     // outputs: with torques the first two components add the derivative recurrence over their b, a warp
     // per (component, parity); the others are spread over the remaining warps
     const bool keep = L.col >= 0 && !L.nyq;
@@ -301,7 +283,7 @@ __global__ void __launch_bounds__((TQ ? 20 : 12) * 32) fold_fwd_kernel(const __g
 // backward: node values on the occupied planes of the DP velocity plus the wall correction (coefficients
 // ecf of e^{-k zeta} and zeta e^{-k zeta}) and, with CURL, the half-curl from the coefficients' derivatives;
 // times 1/(Nx Ny)
-template <typename T, bool CURL, int HP>
+template <bool CURL, int HP>
 __global__ void __launch_bounds__((CURL ? 20 : 12) * 32) fold_bwd_kernel(const __grid_constant__ Geometry g,
                                                                         const T* __restrict__ tab_g,
                                                                         const double2* __restrict__ ecf, int64_t KP,
@@ -316,11 +298,11 @@ __global__ void __launch_bounds__((CURL ? 20 : 12) * 32) fold_bwd_kernel(const _
   const int N = g.nz, M = (N - 1) / 2;
   T* sx = reinterpret_cast<T*>(smraw);  // [NF][N][32]
   T* tab = sx + (size_t)NF * N * 32;
-  T* dn = tab + fold_table_values<T>(N);  // [N] 2 (n + 1) d/dz s, times the half of the curl forward
+  T* dn = tab + fold_table_values(N);  // [N] 2 (n + 1) d/dz s
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, part = lane >> 4, kc = lane & 15;
-  const int nt = (int)fold_table_values<T>(N);
+  const int nt = (int)fold_table_values(N);
   for (int i = threadIdx.x; i < nt; i += NW * 32) tab[i] = tab_g[i];
-  for (int i = threadIdx.x; i < N; i += NW * 32) dn[i] = (T)(1.0 * (2 * (i + 1)) * g.sH);
+  for (int i = threadIdx.x; i < N; i += NW * 32) dn[i] = 2.0 * (i + 1) * g.sH;
   const int64_t K = (int64_t)g.nkx * g.ny, total = (int64_t)w * g.ny;
   const size_t plane = (size_t)g.ny * g.pitch, fs = 2 * (size_t)g.nz * plane;
   const int clo = zrange[0], chi = zrange[1];
@@ -378,7 +360,7 @@ __global__ void __launch_bounds__((CURL ? 20 : 12) * 32) fold_bwd_kernel(const _
       }
     }
     if (CURL) __syncthreads();
-    fold_apply<T, HP>(sx, tab, N);
+    fold_apply<HP>(sx, tab, N);
     T* out = reinterpret_cast<T*>(grid) + 2 * (L.col < 0 ? 0 : L.col) + part;
     for (int c = clo + wi; c <= chi; c += NW) {
       T v[5];
@@ -402,10 +384,9 @@ __global__ void __launch_bounds__((CURL ? 20 : 12) * 32) fold_bwd_kernel(const _
 }
 
 // the parts' matrices, a padded row of outputs per input, times s
-template <typename T>
 std::vector<T> fold_table(int N, double s) {
-  const int n1 = N - 1, h = n1 / 4, k = h / 2, pad = fold_pad<T>(fold_bucket(N));
-  std::vector<T> t(fold_table_values<T>(N), (T)0);
+  const int n1 = N - 1, h = n1 / 4, k = h / 2, pad = fold_pad(fold_bucket(N));
+  std::vector<T> t(fold_table_values(N), (T)0);
   for (int r = 0; r < 4; ++r)
     for (int q = 0; q < 2; ++q) {
       const FoldPart p = fold_part_of(r, q, h);
@@ -448,9 +429,9 @@ __global__ void fold_ecf_kernel(Geometry g, const double* __restrict__ zeta, con
   }
 }
 
-template <typename T, bool C, int HP>
+template <bool C, int HP>
 bool fold_allow() {
-  return allow_smem(fold_fwd_kernel<T, C, HP>) && allow_smem(fold_bwd_kernel<T, C, HP>);
+  return allow_smem(fold_fwd_kernel<C, HP>) && allow_smem(fold_bwd_kernel<C, HP>);
 }
 
 template <typename F>
@@ -480,6 +461,10 @@ bool cheb_fold_applies(const Geometry& g, int precision) {
 //   129 nodes 8: 0.61 / 0.85.  Walls and curls cost the dense kernel terms for all nodes: 65 nodes 1.07 and up
 //   with either; 97 nodes 0.83 with curl, 0.97 with walls, 1.09 with both; 121 nodes 16: bottom wall and curl 0.89,
 //   two walls and curl 1.04; 129 nodes (per-thread kernel) 0.39 to 0.96 at 8, in free space with curl 0.76 at 16.
+// Whole products of a sheet in a box 40 high (folded alone -> this): 256 x 256 x 129 with torques 5.52 -> 2.81 ms,
+// 256 x 256 x 65 forces only 1.51 -> 1.02 ms.  The second launch costs 5 us.  The dense sums inside these kernels
+// instead were up to three times slower backward (their table from global memory, few warps) and took registers
+// from the folded form.
 int fold_thin_planes(const Geometry& g, bool backward) {
   const int N = g.nz;
   if (!backward) return 9 + N / 10;
@@ -493,22 +478,21 @@ int fold_thin_planes(const Geometry& g, bool backward) {
 
 size_t cheb_fold_bytes(const Geometry& g) {
   const size_t KP = (size_t)g.nkx * (g.ny / 2 + 1);
-  return 2 * fold_table_values<double>(g.nz) * sizeof(double) + (g.mode != DPS_FREE ? KP * g.nz * sizeof(double2) : 0);
+  return 2 * fold_table_values(g.nz) * sizeof(double) + (g.mode != DPS_FREE ? KP * g.nz * sizeof(double2) : 0);
 }
 
 dps_status cheb_fold_prepare(Plan& p) {
-  using T = double;
   const Geometry& g = p.g;
   const bool ok = fold_dispatch(fold_bucket(g.nz), [&](auto hp) {
     constexpr int HP = decltype(hp)::value;
-    return g.spectral_curl ? fold_allow<T, true, HP>() : fold_allow<T, false, HP>();
+    return g.spectral_curl ? fold_allow<true, HP>() : fold_allow<false, HP>();
   });
   if (!ok) return DPS_ERR_CUDA;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device) != cudaSuccess) return DPS_ERR_CUDA;
   const int nf = g.spectral_curl ? 5 : 3;
-  p.fold_grid = sms * (2 * (fold_smem<T>(g.nz, nf) + 1024) <= 228 * 1024 && nf == 3 ? 2 : 1);
-  const size_t nt = fold_table_values<T>(g.nz), bytes = cheb_fold_bytes(g);
+  p.fold_grid = sms * (2 * (fold_smem(g.nz, nf) + 1024) <= 228 * 1024 && nf == 3 ? 2 : 1);
+  const size_t nt = fold_table_values(g.nz), bytes = cheb_fold_bytes(g);
   void* q = nullptr;
   if (cudaMalloc(&q, bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -517,7 +501,7 @@ dps_status cheb_fold_prepare(Plan& p) {
   p.kt.fold = reinterpret_cast<double*>(q);
   for (int d = 0; d < 2; ++d) p.fold_thin[d] = fold_thin_planes(g, d == 1);
   p.device_bytes += (int64_t)bytes;
-  const std::vector<T> f = fold_table<T>(g.nz, 2.0 / (g.nz - 1)), b = fold_table<T>(g.nz, 1.0 / ((double)g.nx * (double)g.ny));
+  const std::vector<T> f = fold_table(g.nz, 2.0 / (g.nz - 1)), b = fold_table(g.nz, 1.0 / ((double)g.nx * (double)g.ny));
   if (cudaMemcpy(p.kt.fold, f.data(), nt * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(p.kt.fold + nt, b.data(), nt * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess)
     return DPS_ERR_CUDA;
@@ -531,15 +515,14 @@ dps_status cheb_fold_prepare(Plan& p) {
 }
 
 void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t s) {
-  using T = double;
   const Geometry& g = p.g;
   const int64_t tiles = ((int64_t)w * g.ny + kFoldK - 1) / kFoldK;
-  const size_t nt = fold_table_values<T>(g.nz);
+  const size_t nt = fold_table_values(g.nz);
   cplx<T>* grid = reinterpret_cast<cplx<T>*>(p.grid);
   cplx<T>* kbuf = reinterpret_cast<cplx<T>*>(p.kt.kbuf);
   const cplx<T>* kaux = reinterpret_cast<const cplx<T>*>(p.kt.kaux);
   const int nf = g.spectral_curl ? 5 : 3;
-  const size_t smem = fold_smem<T>(g.nz, nf);
+  const size_t smem = fold_smem(g.nz, nf);
   const unsigned blocks = (unsigned)(tiles < p.fold_grid ? tiles : p.fold_grid);
   const double2* ecf = g.mode != DPS_FREE ? reinterpret_cast<const double2*>(p.kt.fold + 2 * nt) : nullptr;
   const int64_t KP = (int64_t)g.nkx * (g.ny / 2 + 1);
@@ -549,14 +532,14 @@ void launch_cheb_fold(const Plan& p, bool backward, int kx0, int w, cudaStream_t
     constexpr int HP = decltype(hp)::value;
     const int th = 32 * 4 * nf;
     if (!backward && g.spectral_curl)
-      fold_fwd_kernel<T, true, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy, thin);
+      fold_fwd_kernel<true, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy, thin);
     else if (!backward)
-      fold_fwd_kernel<T, false, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy, thin);
+      fold_fwd_kernel<false, HP><<<blocks, th, smem, s>>>(g, p.kt.fold, grid, kbuf, p.zrange, kx0, w, hx, hy, thin);
     else if (g.spectral_curl)
-      fold_bwd_kernel<T, true, HP><<<blocks, th, smem, s>>>(g, p.kt.fold + nt, ecf, KP, kbuf, kaux, grid, p.zrange, kx0, w,
+      fold_bwd_kernel<true, HP><<<blocks, th, smem, s>>>(g, p.kt.fold + nt, ecf, KP, kbuf, kaux, grid, p.zrange, kx0, w,
                                                            hx, hy, thin);
     else
-      fold_bwd_kernel<T, false, HP><<<blocks, th, smem, s>>>(g, p.kt.fold + nt, ecf, KP, kbuf, kaux, grid, p.zrange, kx0,
+      fold_bwd_kernel<false, HP><<<blocks, th, smem, s>>>(g, p.kt.fold + nt, ecf, KP, kbuf, kaux, grid, p.zrange, kx0,
                                                             w, hx, hy, thin);
   });
 }

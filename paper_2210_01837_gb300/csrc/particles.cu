@@ -180,12 +180,12 @@ __device__ __forceinline__ int rec_zsupport(const Geometry& g, const EsKernel& k
 // idle lanes at the images and the shorter supports.  Against a thread per particle: 100 spheres in double 75 ->
 // 14 us, 1001 with torques 92 -> 20, 317 mixed 25 -> 12, 16384 in double 205 -> 172, 16384 mixed 43 -> 27, 262144
 // with derivatives 315 -> 209.
-constexpr int kRecThreads = 128, kRecMax = 32, kRecNodes = 512;  // kRecNodes: nodes copied to shared memory
+constexpr int kRecThreads = 128, kRecMax = 32;
 
 // doubles of a particle's running offsets in shared memory (odd: consecutive particles in different banks)
 __host__ __device__ inline int rec_offsets(const Geometry& g) { return 2 * g.pxc + 1; }
 __host__ __device__ inline size_t rec_smem(const Geometry& g, int P) {
-  return ((size_t)(g.nz <= kRecNodes ? g.nz : 0) + (size_t)P * (g.nkernels * rec_offsets(g) + 3)) * sizeof(double) +
+  return ((size_t)g.nz + (size_t)P * (g.nkernels * rec_offsets(g) + 3)) * sizeof(double) +
          (size_t)2 * P * g.nkernels * sizeof(int);
 }
 
@@ -202,12 +202,10 @@ __global__ void __launch_bounds__(kRecThreads) records_kernel(Geometry g, int64_
   double* offs = rec_sm;                     // [nk][P][no] x offsets, then y offsets
   double* zz3 = offs + (size_t)nk * P * no;  // [P][3] z and its images at the walls
   double* zn = zz3 + 3 * P;                  // [nz] the nodes
-  int* c0s = reinterpret_cast<int*>(zn + (g.nz <= kRecNodes ? g.nz : 0));  // [nk][P] first node
+  int* c0s = reinterpret_cast<int*>(zn + g.nz);  // [nk][P] first node
   int* cnts = c0s + nk * P;                                                // [nk][P] nodes; -1: not in the domain
   const int64_t j0 = (int64_t)blockIdx.x * P;
-  if (g.nz <= kRecNodes)
-    for (int i = tid; i < g.nz; i += kRecThreads) zn[i] = zc_g[i];
-  const double* zc = g.nz <= kRecNodes ? zn : zc_g;
+  for (int i = tid; i < g.nz; i += kRecThreads) zn[i] = zc_g[i];
   __syncthreads();
   const int heads = P < kRecMax ? nk : 1;  // threads per particle: one where the FP64 pipe, not latency, is the bound
   int cmin = g.nz, cmax = -1;
@@ -232,7 +230,7 @@ __global__ void __launch_bounds__(kRecThreads) records_kernel(Geometry g, int64_
           ty += g.h;
         }
         int c0;
-        cnt = rec_zsupport(g, k, zc, a.z, c0, status);
+        cnt = rec_zsupport(g, k, zn, a.z, c0, status);
         hd = make_int4(wrap_idx(ax, g.nx), wrap_idx(ay, g.ny), c0, cnt);
         if (cnt > 0) {
           cmin = min(cmin, c0);
@@ -288,7 +286,7 @@ __global__ void __launch_bounds__(kRecThreads) records_kernel(Geometry g, int64_
     each(g.lzc, [&](int p, int i, T* ph) {
       T v = (T)0, d = (T)0;
       if (i < cnts[K * P + p]) {
-        const double zz = zc[c0s[K * P + p] + i], t = zz - zz3[3 * p];
+        const double zz = zn[c0s[K * P + p] + i], t = zz - zz3[3 * p];
         v = es_t<T>(t, k);
         if (deriv) d = esd_t<T>(t, k);
         if (bottom_img) {

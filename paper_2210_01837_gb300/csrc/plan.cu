@@ -53,7 +53,7 @@ bool fft_plan(int n, FftPlan& fp) {
 
 // Balanced factorisation (the register-staged passes, one butterfly per thread and stage, so their
 // thread count is n / (smallest radix)): the fewest stages, then the largest smallest radix, radices
-// in descending order.  768 = 12 8 8 instead of 16 16 3, 384 = 12 8 4 instead of 16 12 2.
+// in descending order.  768 = 12 8 8 instead of 16 16 3, 384 = 8 8 6 instead of 16 12 2.
 namespace {
 const int kRadices[] = {16, 15, 14, 12, 10, 9, 8, 7, 6, 5, 4, 3, 2};
 void balanced_search(int m, int from, int* cur, int depth, int* best, int& best_depth, int& best_min) {

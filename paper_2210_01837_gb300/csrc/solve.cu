@@ -254,8 +254,6 @@ __device__ __forceinline__ double sweeps(int il, int par, const Rows<T>& tb, con
   return fma(c0, w0, q) + a;
 }
 
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
 // k = 0 (Sec. III.C, Eqs. 47-52; Appendix A, Eq. A12) by one warp, the rows over its lanes; the same
 // rows as zero_mode of the thread-per-wavenumber solves.
 template <typename T, bool SLIP>
