@@ -690,7 +690,8 @@ def main():
                            "frac_fp64_nominal": round(solve_tflops / FP64_NOMINAL_TFLOPS, 3)}
     dom = max((k for k in stages if k in work or k == "solve"), key=stages.get)
     if dom == "solve":
-        roofline = {"bound": "alu", "kernel": "solve_tile_kernel (banded solves)", "achieved": round(solve_tflops, 4),
+        roofline = {"bound": "alu", "kernel": "solve_tile_kernel (banded solves)" if not args.nz else "banded solves",
+                    "achieved": round(solve_tflops, 4),
                     "peak": round(FP64_NOMINAL_TFLOPS, 3), "unit": "TFLOP/s",
                     "frac": round(solve_tflops / FP64_NOMINAL_TFLOPS, 4),
                     "traffic": measured_traffic("solve_tile_kernel<float, 0>") if div == 1 and not args.nz else None,
