@@ -148,7 +148,11 @@ __global__ void __launch_bounds__(kColThreads, col_blocks(HP)) cols_bwd_kernel(c
         }
       }
       const double hx = hpx * (double)L.kxi, hy = hpy * (double)L.nyv;
-      kk = 2.0f * sqrtf((float)(hx * hx + hy * hy));
+      // |k| = 2 sqrt(s) as a square root in double, rounded to float, gives it, without holding up the FP64
+      // pipe: a float root and one Newton step with the residual formed in double
+      const double s = hx * hx + hy * hy;
+      const float r = sqrtf(d2f(s));
+      if (r > 0.f) kk = fmaf(2.0f, r, __fdividef(d2f(fma(-f2d(r), f2d(r), s)), r));
     }
     for (int c = 0; c < np; ++c) {
       const int m = n1 - c;
