@@ -200,6 +200,16 @@ __device__ __forceinline__ void functionals(int il, const Rows<T>& tb, double* s
   });
 }
 
+// a coefficient in the transform precision, to nearest (narrow truncates; these enter the output)
+__device__ __forceinline__ void round_to(double d, double& v) { v = d; }
+__device__ __forceinline__ void round_to(double d, float& v) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned s = hi & 0x80000000u;
+  const int e = (int)((hi >> 20) & 0x7ffu) - 896;
+  const unsigned m = ((unsigned)e << 23 | (hi & 0xfffffu) << 3 | lo >> 29) + (lo >> 28 & 1u);  // may carry into e
+  v = __uint_as_float(s | (e <= 0 ? 0u : e >= 255 ? 0x7f800000u : m));
+}
+
 // Passes 2 and 3 of a system: the elimination in place and s_1 from it, the 2 x 2 boundary system for c_0 and
 // a, and the substitution c_i = s_i - t_i c_{i-1} with y = B B c (+ a in row 0) handed to put(i, y) in the
 // transform precision.  Returns the wall value's and (qd) the wall derivative's part of this parity.
@@ -232,8 +242,9 @@ __device__ __forceinline__ double sweeps(int il, int par, const Rows<T>& tb, con
   });
   const double rh = fma(-s, U, widen<T>(r0));
   const double c0 = fma(g, ck, rh * cb), a = fma(g, cd, -(rh * cc));
-  const T ta = narrow<T>(a);
-  T c2 = (T)0, c1 = narrow<T>(c0);
+  T ta, c1, c2 = (T)0;
+  round_to(a, ta);
+  round_to(c0, c1);
   auto row = [&](int i, T cn) {  // row i of y, whose neighbours c_{i-1} and c_{i+1} = cn are known now
     const int n = par + 2 * i;
     const T y = (c1 * m.td[n] + cn * m.tu[n]) + c2 * m.tl[n];  // c2 = 0 in row 0
@@ -244,7 +255,9 @@ __device__ __forceinline__ double sweeps(int il, int par, const Rows<T>& tb, con
   double c = c0;
   rows_ahead<4, 1, double>(t, 1, il, ft, [&](int i, double f) {
     c = fma(f, c, sw[i * 32]);
-    row(i - 1, narrow<T>(c));
+    T cn;
+    round_to(c, cn);
+    row(i - 1, cn);
   });
   row(il, (T)0);
   if (SLIP) {
