@@ -403,26 +403,33 @@ std::vector<T> fold_table(int N, double s) {
   return t;
 }
 
-// coefficients of e^{-k zeta} and zeta e^{-k zeta} per (kx, |ky|): a block per kp, a thread per coefficient
-__global__ void fold_ecf_kernel(Geometry g, const double* __restrict__ zeta, const double* __restrict__ cmat, int64_t KP,
-                                double2* __restrict__ ecf) {
-  extern __shared__ double sm[];
-  double *e = sm, *z = sm + g.nz;
+// coefficients of e^{-k zeta} and zeta e^{-k zeta} per (kx, |ky|): a block per kp, a thread per coefficient, from
+// the sums (even coefficients) and differences (odd) of mirrored nodes.  ct: [node][coefficient], so that a
+// warp reads a row of it.
+__global__ void fold_ecf_kernel(Geometry g, const double* __restrict__ zeta, const double* __restrict__ ct, int npad,
+                                int64_t KP, double2* __restrict__ ecf) {
+  extern __shared__ double2 ecf_sm[];
+  const int N = g.nz, half = (N + 1) / 2;
+  double2 *sum = ecf_sm, *dif = ecf_sm + half;  // [half] of both functions; the middle node (N odd) counts once
   for (int64_t kp = blockIdx.x; kp < KP; kp += gridDim.x) {
     const int kxi = (int)(kp % g.nkx), kyi = (int)(kp / g.nkx);
     const double kx = 2.0 * M_PI * (double)kxi / g.Lx, ky = 2.0 * M_PI * (double)kyi / g.Ly;
     const double kk = sqrt(kx * kx + ky * ky);
     __syncthreads();
-    for (int c = threadIdx.x; c < g.nz; c += blockDim.x) {
-      e[c] = exp(-kk * zeta[c]);
-      z[c] = zeta[c] * e[c];
+    for (int c = threadIdx.x; c < half; c += blockDim.x) {
+      const double za = zeta[c], zb = zeta[N - 1 - c], a = exp(-kk * za), b = exp(-kk * zb);
+      const bool mid = c == N - 1 - c;
+      sum[c] = mid ? make_double2(a, za * a) : make_double2(a + b, za * a + zb * b);
+      dif[c] = mid ? make_double2(0.0, 0.0) : make_double2(a - b, za * a - zb * b);
     }
     __syncthreads();
-    for (int n = threadIdx.x; n < g.nz; n += blockDim.x) {
+    for (int n = threadIdx.x; n < N; n += blockDim.x) {
+      const double2* f = n & 1 ? dif : sum;
       double a = 0.0, b = 0.0;
-      for (int c = 0; c < g.nz; ++c) {
-        a = fma(cmat[(size_t)n * g.nz + c], e[c], a);
-        b = fma(cmat[(size_t)n * g.nz + c], z[c], b);
+      for (int c = 0; c < half; ++c) {
+        const double w = ct[(size_t)c * npad + n];
+        a = fma(w, f[c].x, a);
+        b = fma(w, f[c].y, b);
       }
       ecf[(size_t)n * KP + kp] = make_double2(a, b);
     }
@@ -507,8 +514,8 @@ dps_status cheb_fold_prepare(Plan& p) {
     return DPS_ERR_CUDA;
   if (g.mode != DPS_FREE) {
     const int64_t KP = (int64_t)g.nkx * (g.ny / 2 + 1);
-    fold_ecf_kernel<<<(unsigned)(KP < 152 * 16 ? KP : 152 * 16), 128, 2 * g.nz * sizeof(double)>>>(
-        g, reinterpret_cast<const double*>(p.tab.zeta), reinterpret_cast<const double*>(p.kt.cmat), KP,
+    fold_ecf_kernel<<<(unsigned)(KP < sms * 16 ? KP : sms * 16), 128, (g.nz + 1) / 2 * 2 * sizeof(double2)>>>(
+        g, reinterpret_cast<const double*>(p.tab.zeta), reinterpret_cast<const double*>(p.kt.ct), p.kt.npad, KP,
         reinterpret_cast<double2*>(p.kt.fold + 2 * nt));
   }
   return cudaGetLastError() == cudaSuccess ? DPS_OK : DPS_ERR_CUDA;
