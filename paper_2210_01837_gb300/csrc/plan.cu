@@ -358,30 +358,8 @@ dps_status allocate(Plan* p) {
   }
   if (!alloc((void**)&p->stage_in, nmax * 9 * sizeof(double))) return DPS_ERR_OOM;
   if (!alloc((void**)&p->stage_out, nmax * 6 * sizeof(double))) return DPS_ERR_OOM;
-  if (!fft_rows_allow<T>() || !fft_cols_allow<T>() || !fft_rows_default<T>(*p) || !fft_cols_default<T>(*p))
-    return DPS_ERR_INVALID_ARG;
-  const int sp = spread_prepare<T>(*p);
-  if (sp < 0) return DPS_ERR_INVALID_ARG;
-  if (sp == 0) return DPS_ERR_CUDA;
-  // the staged interpolation's TMA view of the grid (without it every bin copies with cp.async)
-  p->interp_tma = interp_stage_fields(g, (int)(sizeof(T) / 4)) > 0 && encode_interp_tmap(*p) ? 1 : 0;
-  // column chunks of the wavenumber-space pipeline (multiples of 32 columns, ~192 wide)
-  // one chunk by default: measured on GB300, co-running the FP64 solve with the float transforms
-  // slowed both (they compete for issue slots); DPS_CHUNKS in the environment or the autotuner may
-  // choose more
-  int J = 1;
-  if (const char* e = getenv("DPS_CHUNKS")) J = std::max(1, std::min(atoi(e), kMaxChunks));
-  if (!set_chunks(*p, J)) set_chunks(*p, 1);
-  for (int i = 0; i < 2; ++i)
-    if (cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) != cudaSuccess) return DPS_ERR_CUDA;
-  if (cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
-  for (int j = 0; j < kMaxChunks; ++j) {  // events for every chunk count the autotuner may pick
-    if (cudaEventCreateWithFlags(&p->ev_f[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
-    if (cudaEventCreateWithFlags(&p->ev_s[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
-    if (cudaEventCreateWithFlags(&p->ev_b[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
-  }
-  // Last, what a plan can run without, in the order of its worth, so that scarce memory goes to what it needs:
-  // the solve's table (per (kx, |ky|), filled on the legacy stream; without it the solve factorises as it goes;
+  // After all that, what a plan can run without, in the order of its worth, so that scarce memory goes to what it
+  // needs: the solve's table (per (kx, |ky|), filled on the legacy stream; without it the solve factorises as it goes;
   // DPS_SOLVE_TABLE=0 chooses that by hand) and the folded transforms' tables (without them: dense).  The
   // tiled solve needs its table and no workspace; the thread-per-wavenumber solves need their workspace.
   const int64_t need_blocks = std::max<int64_t>(1, (K + kBvpThreads - 1) / kBvpThreads);
@@ -412,6 +390,28 @@ dps_status allocate(Plan* p) {
     const dps_status fs = cheb_fold_prepare(*p);
     if (fs == DPS_ERR_CUDA) return fs;
     p->cheb_fold = fs == DPS_OK ? 1 : 0;
+  }
+  if (!fft_rows_allow<T>() || !fft_cols_allow<T>() || !fft_rows_default<T>(*p) || !fft_cols_default<T>(*p))
+    return DPS_ERR_INVALID_ARG;
+  const int sp = spread_prepare<T>(*p);
+  if (sp < 0) return DPS_ERR_INVALID_ARG;
+  if (sp == 0) return DPS_ERR_CUDA;
+  // the staged interpolation's TMA view of the grid (without it every bin copies with cp.async)
+  p->interp_tma = interp_stage_fields(g, (int)(sizeof(T) / 4)) > 0 && encode_interp_tmap(*p) ? 1 : 0;
+  // column chunks of the wavenumber-space pipeline (multiples of 32 columns, ~192 wide)
+  // one chunk by default: measured on GB300, co-running the FP64 solve with the float transforms
+  // slowed both (they compete for issue slots); DPS_CHUNKS in the environment or the autotuner may
+  // choose more
+  int J = 1;
+  if (const char* e = getenv("DPS_CHUNKS")) J = std::max(1, std::min(atoi(e), kMaxChunks));
+  if (!set_chunks(*p, J)) set_chunks(*p, 1);
+  for (int i = 0; i < 2; ++i)
+    if (cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) != cudaSuccess) return DPS_ERR_CUDA;
+  if (cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
+  for (int j = 0; j < kMaxChunks; ++j) {  // events for every chunk count the autotuner may pick
+    if (cudaEventCreateWithFlags(&p->ev_f[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
+    if (cudaEventCreateWithFlags(&p->ev_s[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
+    if (cudaEventCreateWithFlags(&p->ev_b[j], cudaEventDisableTiming) != cudaSuccess) return DPS_ERR_CUDA;
   }
   return DPS_OK;
 }
