@@ -12,12 +12,12 @@
 // s - 1, one barrier a step.  Sweep values live in shared memory, so the DRAM traffic falls from 4.8 to
 // 1.3 GB at 768 x 768 x 65 (spectra and table).
 //
-// Measured (solve alone, GB300, thread per wavenumber -> this): 120 x 120 x 33 mixed 155 -> 47 us,
-// 128 x 128 x 65 double 434 -> 172 us, 768 x 768 x 65 mixed 1.72 -> 1.40 ms, 3072 x 3072 x 65 mixed
-// 23.2 -> 22.3 ms.  It is bound by latency: 16 warps an SM (the slabs' shared memory).  The sweeps run in
-// double in float plans too, as the boundary sums do: 64-bit fixed-point sweeps on the integer pipe took the
-// same time (1.40 and 22.3 ms), lost bits in the small entries of a column and turned an overflow into
-// finite numbers.
+// Measured (solve alone, GB300, thread per wavenumber -> this): 120 x 120 x 33 mixed 155 -> 46 us,
+// 128 x 128 x 65 double 434 -> 170 us, 768 x 768 x 65 mixed 1.72 -> 1.38 ms, 3072 x 3072 x 65 mixed
+// 23.2 -> 21.8 ms.  It is bound by the FP64 pipe, 77 % busy there (16 warps an SM, the slabs' shared memory, and
+// a barrier a step leave the rest).  The sweeps run in double in float plans too, as the boundary sums do:
+// 64-bit fixed-point sweeps on the integer pipe took the same time (1.40 and 22.3 ms), lost bits in the small
+// entries of a column and turned an overflow into finite numbers.
 #include "bvp_device.cuh"
 #include "dps_internal.cuh"
 
