@@ -61,3 +61,25 @@ def test_paired_first_and_last_stages_match_oracle(nx):
         plan.close()
         assert rel_l2(U, U_ref) <= TOL[precision], precision
         assert rel_l2(W, W_ref) <= TOL[precision], precision
+
+
+@pytest.mark.parametrize("n", [3430, 3528, 3600, 3840])
+def test_longest_double_sizes_match_oracle(n):
+    """Double rows and columns that only the composite radices fit (3840 = 16 16 15 in 256 threads), in every
+    variant that they have."""
+    for nx, ny in ((n, 16), (16, n)):
+        params = small_params("bottom_wall", nx=nx, ny=ny, nz=9, zmax=4.0, torque=True)
+        pos, F, T = random_particles(params, 12, seed=n)
+        U_ref, W_ref = mobility(oracle_params(params), pos, F, T)
+        plan = binding.Plan.from_params(params, with_torque=True, precision="fp64", max_n=len(pos))
+        info = plan.info()
+        for cols in (info.fft_register_cols,) if nx == n else (1, 2, 3):
+            try:
+                plan.set_fft(info.fft_register_rows, cols, info.fft_col_width)
+            except binding.DpsError:
+                assert cols != info.fft_register_cols
+                continue
+            U, W = gpu_mobility(params, pos, F, T, "fp64", plan=plan)
+            assert rel_l2(U, U_ref) <= TOL["fp64"], (nx, ny, cols)
+            assert rel_l2(W, W_ref) <= TOL["fp64"], (nx, ny, cols)
+        plan.close()
